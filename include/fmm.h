@@ -77,11 +77,13 @@ typedef struct {
                               FMM_F64; the paper suggests 2 for its CPU
                               cluster and tuning per platform, Sec. 5.5);
                               +inf allowed                                     */
-    double bucket;         /* accepted bucket width inside a brick, in units of
-                              h * min(1/F) / sqrt(3); 0 -> 4 (0.6 for the
-                              second-order march, whose accepted values must
-                              be final when their neighbours read them: see
-                              accuracy); +inf allowed                        */
+    double bucket;         /* bucket width of the cell-parallel schedule (4), in
+                              units of h * min(1/F) / sqrt(3); 0 -> 4 (0.6 for
+                              the second-order march, whose accepted values
+                              must be final when their neighbours read them:
+                              see accuracy); +inf allowed.  The brick
+                              schedules sweep a brick in the order of its
+                              cells and take no bucket                       */
     int32_t ctas;          /* CTAs of the march kernel; 0 -> as many as fit     */
     int32_t timeout_s;     /* host wall-clock limit of one solve in seconds;
                               0 -> 600; exceeding it returns FMM_ERR_TIMEOUT  */
@@ -179,7 +181,7 @@ typedef struct {
                                 (schedule 4: bucket steps that accepted
                                 cells; its brick counters stay 0)             */
     int64_t brick_marches;   /* local marches of a brick (both phases)           */
-    int64_t march_rounds;    /* bucket rounds summed over all brick marches      */
+    int64_t march_rounds;    /* sweeps summed over all brick marches             */
     int64_t exchanges;       /* brick faces that sent changed overlap data       */
     int64_t accepted;        /* cell acceptances (re-acceptances counted again)  */
     int64_t n_bricks;        /* bricks of the grid                               */
@@ -208,7 +210,7 @@ typedef struct fmm_handle fmm_handle;
  *                  when n_src == 0.
  *   out          : receives the handle (owned by the caller; fmm_destroy).
  * The handle owns all device workspace (brick-layout psi and tags, per-brick
- * front minima and exchange masks, work lists, the restart control block and,
+ * front minima and work words, work lists, the restart control block and,
  * when record_tape is set, the upwind tape).
  */
 fmm_status fmm_create(const fmm_config *cfg, const void *speed, double speed_const,
@@ -290,7 +292,7 @@ fmm_status fmm_resume(fmm_handle *hd, int64_t more_restarts, void *T_out, uint8_
 
 /*
  * Checkpoints of a solve state, in host memory: the brick-layout psi, tags,
- * tape (when recorded), per-brick BAND minima, halo change masks and dirty
+ * tape (when recorded), per-brick BAND minima, pending halo changes and dirty
  * flags, and the restart control block, after an 88-byte header that records
  * the grid, dtype, cell sizes, record_tape and the kind of speed.
  *   fmm_checkpoint_size -- bytes an image of hd takes (*bytes).

@@ -90,7 +90,7 @@ fmm_status cuda_fail(fmm_handle *hd, cudaError_t e, const char *where)
 void free_state(fmm_handle *hd)
 {
     DeviceState &s = hd->st;
-    void *ptrs[] = {s.T,      s.tag,      s.spd,   s.bdelta,  s.tape,   s.bmin,   s.fresh, s.inmin, s.inbox,
+    void *ptrs[] = {s.T,      s.tag,      s.spd,   s.bdelta,  s.tape,   s.bmin,   s.work, s.waiting,
                     s.dirty,  s.list[0],  s.list[1], s.ctrl,  hd->d_src, s.queue, s.queued, s.faces};
     for (void *p : ptrs)
         if (p)
@@ -263,10 +263,10 @@ fmm_status run_solve(fmm_handle *hd, void *T_out, uint8_t *tags_out)
     cudaStream_t st = hd->stream;
     hd->solved = hd->tape_valid = hd->resumable = hd->complete = false;
     FMM_CUDA(hd, launch_reset_control(s, st, hd->params.wait_ns, hd->params.hold));
-    FMM_CUDA(hd, cudaMemsetAsync(s.fresh, 0, (size_t)g.nbricks * kFaces * sizeof(unsigned long long), st));
-    FMM_CUDA(hd, cudaMemsetAsync(s.inmin, 0xff, (size_t)g.nbricks * 2 * sizeof(unsigned long long), st));
+    FMM_CUDA(hd, cudaMemsetAsync(s.work, 0xff, (size_t)g.nbricks * sizeof(unsigned long long), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.dirty, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
+    FMM_CUDA(hd, cudaMemsetAsync(s.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queued, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, launch_front_init(dt, g, s, hd->params, st));
     return run_restarts(hd, T_out, tags_out, 2);   // control reset, front init
@@ -532,7 +532,9 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
 bool aligned16(const void *p) { return ((uintptr_t)p & 15u) == 0; }
 
 // Checkpoint image: this header, then T, tags, the tape (if recorded), the
-// per-brick BAND minima, the change masks and the dirty flags (the brick
+// per-brick BAND minima, 48 bytes per brick that are zero (images of earlier
+// builds hold masks there, which nothing needs: the values that came with them
+// follow), the smallest changed halo values and the dirty flags (the brick
 // layout of the device), then the control block the forward solve ended with.
 struct CkptHeader {
     char magic[8];
@@ -550,8 +552,9 @@ constexpr char kCkptMagic[8] = {'F', 'M', 'M', 'C', 'K', 'P', 'T', '1'};
 static_assert(sizeof(CkptHeader) == 88, "the header size fmm.h documents");
 
 struct CkptSection {
-    void *dev;
+    void *dev;   // null: a section of zeros
     size_t bytes;
+    bool work = false;   // the work words: the image holds a double per side
 };
 
 std::vector<CkptSection> ckpt_sections(fmm_handle *hd)
@@ -562,8 +565,8 @@ std::vector<CkptSection> ckpt_sections(fmm_handle *hd)
     if (s.tape)
         v.push_back({s.tape, cells});
     v.push_back({s.bmin, 2 * nb * hd->rsize});
-    v.push_back({s.fresh, nb * kFaces * sizeof(unsigned long long)});
-    v.push_back({s.inmin, nb * 2 * sizeof(unsigned long long)});
+    v.push_back({nullptr, nb * kFaces * sizeof(unsigned long long)});
+    v.push_back({s.work, nb * 2 * sizeof(unsigned long long), true});
     v.push_back({s.dirty, nb * sizeof(unsigned)});
     return v;
 }
@@ -705,9 +708,8 @@ fmm_status fmm_create(const fmm_config *cfg, const void *speed, double speed_con
     ALLOC(s.tag, cells);
     ALLOC(s.bdelta, nb * hd->rsize);
     ALLOC(s.bmin, 2 * nb * hd->rsize);
-    ALLOC(s.fresh, nb * kFaces * sizeof(unsigned long long));
-    ALLOC(s.inmin, nb * 2 * sizeof(unsigned long long));
-    ALLOC(s.inbox, nb * kFaces * sizeof(unsigned long long));
+    ALLOC(s.work, nb * sizeof(unsigned long long));
+    ALLOC(s.waiting, nb * sizeof(unsigned long long));
     ALLOC(s.dirty, nb * sizeof(unsigned));
     ALLOC(s.list[0], nb * sizeof(int));
     ALLOC(s.list[1], nb * sizeof(int));
@@ -730,7 +732,7 @@ fmm_status fmm_create(const fmm_config *cfg, const void *speed, double speed_con
     if (e != cudaSuccess)
         return bail(cuda_fail(hd, e, "cudaMallocHost"));
     const int per_sm = march_blocks_per_sm(cfg->dtype, cfg->record_tape != 0);
-    s.march_ctas = cfg->ctas > 0 ? cfg->ctas : sms * per_sm;
+    s.march_ctas = cfg->ctas > 0 ? cfg->ctas : march_grid(sms * per_sm, g.nbricks);
     hd->params.raise_at = raise_threshold(s.march_ctas);
     fmm_status rc = load_speed(hd, speed, speed_const);
     if (rc != FMM_OK)
@@ -904,6 +906,9 @@ fmm_status fmm_resume(fmm_handle *hd, int64_t more_restarts, void *T_out, uint8_
     hd->pre_launches = 0;
     cudaError_t e = cudaMemcpyAsync(hd->st.ctrl, hd->h_ctrl, sizeof(Control), cudaMemcpyHostToDevice,
                                     hd->stream);
+    // (a launch stopped by its restart limit leaves entries in the waiting ring)
+    if (e == cudaSuccess)
+        e = cudaMemsetAsync(hd->st.waiting, 0, (size_t)hd->geom.nbricks * sizeof(unsigned long long), hd->stream);
     if (e == cudaSuccess && hd->st.faces)
         e = launch_faces_build(hd->cfg.dtype, hd->geom, hd->st, hd->stream);   // from the stopped state
     if (e != cudaSuccess) {
@@ -969,10 +974,10 @@ fmm_status fmm_dd_start(fmm_handle *hd, const void *phi0, int64_t extra_lo, int6
     }
     hd->solved = hd->tape_valid = hd->resumable = hd->complete = false;
     FMM_CUDA(hd, launch_reset_control(s, st, hd->params.wait_ns, hd->params.hold));
-    FMM_CUDA(hd, cudaMemsetAsync(s.fresh, 0, (size_t)g.nbricks * kFaces * sizeof(unsigned long long), st));
-    FMM_CUDA(hd, cudaMemsetAsync(s.inmin, 0xff, (size_t)g.nbricks * 2 * sizeof(unsigned long long), st));
+    FMM_CUDA(hd, cudaMemsetAsync(s.work, 0xff, (size_t)g.nbricks * sizeof(unsigned long long), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.dirty, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
+    FMM_CUDA(hd, cudaMemsetAsync(s.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queued, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, launch_front_init(dt, g, s, hd->params, st));
     FMM_CUDA(hd, cudaStreamSynchronize(st));
@@ -1101,7 +1106,25 @@ fmm_status fmm_checkpoint_save(fmm_handle *hd, void *host_buf, int64_t capacity)
     memcpy(p, &hdr, sizeof(hdr));
     p += sizeof(hdr);
     for (const CkptSection &c : ckpt_sections(hd)) {
-        FMM_CUDA(hd, cudaMemcpy(p, c.dev, c.bytes, cudaMemcpyDeviceToHost));
+        if (c.work) {
+            // (the smallest work of a brick as a double, on one side; all ones: none)
+            std::vector<unsigned long long> w(c.bytes / 16);
+            FMM_CUDA(hd, cudaMemcpy(w.data(), c.dev, c.bytes / 2, cudaMemcpyDeviceToHost));
+            for (size_t b = 0; b < w.size(); ++b) {
+                const unsigned k = (unsigned)(w[b] >> 32);
+                unsigned long long out[2] = {~0ull, ~0ull};
+                if (k < 0x7f800000u) {
+                    float f;
+                    memcpy(&f, &k, sizeof(f));
+                    const double d = f;
+                    memcpy(&out[1], &d, sizeof(d));
+                }
+                memcpy(p + 16 * b, out, sizeof(out));
+            }
+        } else if (c.dev)
+            FMM_CUDA(hd, cudaMemcpy(p, c.dev, c.bytes, cudaMemcpyDeviceToHost));
+        else
+            memset(p, 0, c.bytes);
         p += c.bytes;
     }
     memcpy(p, &hd->fwd_ctrl, sizeof(Control));
@@ -1131,7 +1154,26 @@ fmm_status fmm_checkpoint_load(fmm_handle *hd, const void *host_buf, int64_t siz
     FMM_CUDA(hd, cudaStreamSynchronize(hd->stream));
     const unsigned char *p = (const unsigned char *)host_buf + sizeof(hdr);
     for (const CkptSection &c : ckpt_sections(hd)) {
-        FMM_CUDA(hd, cudaMemcpy(c.dev, p, c.bytes, cudaMemcpyHostToDevice));
+        if (c.work) {
+            std::vector<unsigned long long> w(c.bytes / 16);
+            for (size_t b = 0; b < w.size(); ++b) {
+                unsigned long long in[2];
+                memcpy(in, p + 16 * b, sizeof(in));
+                float f = INFINITY;
+                for (unsigned long long bits : in)
+                    if (bits < 0x7ff0000000000000ull) {
+                        double d;
+                        memcpy(&d, &bits, sizeof(d));
+                        const float r = (float)d;
+                        f = std::fmin(f, (double)r > d ? std::nextafter(r, 0.0f) : r);
+                    }
+                unsigned k;
+                memcpy(&k, &f, sizeof(k));
+                w[b] = (unsigned long long)k << 32;
+            }
+            FMM_CUDA(hd, cudaMemcpy(c.dev, w.data(), c.bytes / 2, cudaMemcpyHostToDevice));
+        } else if (c.dev)
+            FMM_CUDA(hd, cudaMemcpy(c.dev, p, c.bytes, cudaMemcpyHostToDevice));
         p += c.bytes;
     }
     memcpy(&hd->fwd_ctrl, p, sizeof(Control));
@@ -1143,6 +1185,7 @@ fmm_status fmm_checkpoint_load(fmm_handle *hd, const void *host_buf, int64_t siz
     // the queue is empty between restarts
     const Geom &g = hd->geom;
     FMM_CUDA(hd, cudaMemset(hd->st.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long)));
+    FMM_CUDA(hd, cudaMemset(hd->st.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long)));
     FMM_CUDA(hd, cudaMemset(hd->st.queued, 0, (size_t)g.nbricks * sizeof(unsigned)));
     hd->complete = hdr.complete != 0;
     hd->resumable = hdr.resumable != 0;
@@ -1276,9 +1319,8 @@ fmm_status fmm_create_batch(int n_grids, const int64_t *dims, const double *h,
     ALLOC(s.spd, cells * hd->rsize);
     ALLOC(s.bdelta, nb * hd->rsize);
     ALLOC(s.bmin, 2 * nb * hd->rsize);
-    ALLOC(s.fresh, nb * kFaces * sizeof(unsigned long long));
-    ALLOC(s.inmin, nb * 2 * sizeof(unsigned long long));
-    ALLOC(s.inbox, nb * kFaces * sizeof(unsigned long long));
+    ALLOC(s.work, nb * sizeof(unsigned long long));
+    ALLOC(s.waiting, nb * sizeof(unsigned long long));
     ALLOC(s.dirty, nb * sizeof(unsigned));
     ALLOC(s.list[0], nb * sizeof(int));
     ALLOC(s.list[1], nb * sizeof(int));
@@ -1297,7 +1339,7 @@ fmm_status fmm_create_batch(int n_grids, const int64_t *dims, const double *h,
     memcpy(hd->h_grids, grids.data(), (size_t)n_grids * sizeof(BatchGrid));
     s.nbr = hd->d_nbr;
     const int per_sm = march_blocks_per_sm(cfg->dtype, false);
-    s.march_ctas = cfg->ctas > 0 ? cfg->ctas : sms * per_sm;
+    s.march_ctas = cfg->ctas > 0 ? cfg->ctas : march_grid(sms * per_sm, g.nbricks);
     hd->params.raise_at = raise_threshold(s.march_ctas);
     e = cudaMemcpy(hd->d_nbr, nbr.data(), nb * kFaces * sizeof(int), cudaMemcpyHostToDevice);
     if (e == cudaSuccess)

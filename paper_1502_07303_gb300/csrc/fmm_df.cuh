@@ -189,4 +189,128 @@ __device__ __forceinline__ int df_shifted_root(double m, double v1, double v2, i
     return 0;
 }
 
+// sqrt and reciprocal estimates (about one float ulp; subnormals count as 0,
+// sqrt(+inf) = +inf, a negative argument gives NaN)
+__device__ __forceinline__ float sqrt_est(float x)
+{
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float rcp_est(float x)
+{
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+// A non-negative double as a double-float: the top 24 significant bits and
+// the remaining 29 fraction bits, which the conversion rounds to 24.  The
+// magnitude is clamped to [2^-100, 2^96] on the exponent (+inf comes out as
+// 2^96); below 2^-74 the low part is only an error of at most 2^-97.
+__device__ __forceinline__ dfl df_split(double v)
+{
+    const unsigned lo = (unsigned)__double2loint(v);
+    const unsigned hi = umin(umax((unsigned)__double2hiint(v), 923u << 20), 1119u << 20);
+    // 2^(E - 1075), the weight of the last fraction bit
+    const float ulp = __uint_as_float(((umax(hi, 949u << 20) - (948u << 20)) & 0x7ff00000u) << 3);
+    return {__uint_as_float(__funnelshift_l(lo, hi - (896u << 20), 3)),
+            __uint2float_rn(lo & 0x1fffffffu) * ulp};
+}
+
+// u0 + c as a double, |c| below 1e-6 u0: the bit pattern of u0 moved by c in
+// units of four last places (the patterns of adjacent doubles are adjacent
+// integers), so no FP64 addition is spent.  A sum that leaves u0's binade
+// counts the units beyond it double (below) or half (above).
+// c2 is a second, smaller part of c.
+__device__ __forceinline__ double df_shift(float u0, float c, float c2 = 0.0f)
+{
+    const unsigned E = (__float_as_uint(u0) >> 23) & 0xffu;
+    const float inv = __uint_as_float((304u - E) << 23);   // 2^(50 - (E - 127))
+    const long long d = 4ll * (__float2int_rn(c * inv) + (c2 != 0.0f ? __float2int_rn(c2 * inv) : 0));
+    const long long base = (long long)(E + 896u) << 52;
+    const long long f = ((long long)(__float_as_uint(u0) & 0x7fffffu) << 29) + d;   // fraction field
+    long long t = base + f;
+    if ((unsigned)((unsigned long long)f >> 32) >> 20)
+        t += f < 0 ? f : -((f - (1ll << 52)) >> 1);
+    return __longlong_as_double(t);
+}
+
+// What df_root needs of a speed term q = (h/F)^2 in [1e-30, 1e30]: q as a
+// double-float, its square root, 2 q and 3 q.
+struct DfSpeed {
+    float h, l, s, h2, h3;
+};
+__device__ __forceinline__ DfSpeed df_speed(double q)
+{
+    const dfl Q = df_split(q);
+    return {Q.h, Q.l, sqrt_est(Q.h), 2.0f * Q.h, 3.0f * Q.h};
+}
+
+// Algorithm 11's root for sorted upwind values m <= v1 <= v2 (+inf: absent; m
+// finite), t = m + u as above: the upwind set and a root u0 in float, then the
+// exact root of the quadratic about u0.
+//
+// The set grows while its root exceeds the next shift (the root of the larger
+// set is below that of the smaller one and above the shift it added).  In
+// float these tests can err where a root and a shift agree to about 1e-7; the
+// two sets' roots then differ by about 1e-14 u, so without a recorded set
+// either will do.  kStrict (the set is recorded): a test closer than 1e-5 goes
+// to df_shifted_root, which decides on the doubles the cells hold.
+//
+// With r = q - sum (u0 - delta_i)^2 in double-float and g = sum (u0 -
+// delta_i), u - u0 = c - k c^2 / (2 g) + O(c^3), c = r / (2 g); c is about 1e-7
+// u0, so its float rounding is below 1e-14 u0.  Three FP64 additions in all
+// (two shifts and m + u) on a pipe that takes one warp instruction in 16
+// cycles, against four, and about half the float operations, when the root is
+// carried in double-float throughout (df_shifted_root).
+template <bool kStrict>
+__device__ __forceinline__ int df_root(double m, double v1, double v2, const DfSpeed &Q, double q, double &t)
+{
+    const dfl D1 = df_split(v1 - m), D2 = df_split(v2 - m);
+    const float a1 = D1.h, a2 = D2.h, e = a2 - a1, f1 = a1 * a1;
+    const bool c1 = a1 < Q.s;
+    const float u2 = c1 ? 0.5f * (a1 + sqrt_est(Q.h2 - f1)) : Q.s;
+    const bool c2 = a2 < u2;
+    if constexpr (kStrict) {
+        if (fabsf(a1 - Q.s) < 1e-5f * Q.s || (c1 && fabsf(a2 - u2) < 1e-5f * u2))
+            return df_shifted_root<true>(m, v1, v2, v1 < 1e300 ? (v2 < 1e300 ? 3 : 2) : 1, q, t);
+    }
+    // (products that feed an error-free sum are rounded on their own: a fused
+    // multiply-add there would not be the sum whose error is taken)
+    const float u0 = c2 ? __fmul_rn((a1 + a2) + sqrt_est(Q.h3 - fmaf(a2, a2, fmaf(e, e, f1))), 0.333333343f) : u2;
+    // u0 - delta_i as high + low parts (0 for an axis that is not in the
+    // set; u0 is not below a shift of the set, so the difference's error is
+    // the two-term one)
+    const float b1 = c1 ? a1 : u0, b2 = c2 ? a2 : u0;
+    const float x1 = u0 - b1, x2 = u0 - b2;
+    const float l1 = ((u0 - x1) - b1) - (c1 ? D1.l : 0.0f), l2 = ((u0 - x2) - b2) - (c2 ? D2.l : 0.0f);
+    // r: every partial sum is at least what is subtracted next
+    const float p0 = __fmul_rn(u0, u0), p1 = __fmul_rn(x1, x1);
+    const float s0 = Q.h - p0, s1 = s0 - p1;
+    const float r0 = ((Q.h - s0) - p0) - fmaf(u0, u0, -p0);
+    const float r1 = ((s0 - s1) - p1) - fmaf(x1, x1, -p1);
+    const float z = fmaf(x1, l1, x2 * l2);
+    const float ra = fmaf(-x2, x2, s1), rb = fmaf(-2.0f, z, (r0 + r1) + Q.l);
+    const float g = u0 + (x1 + x2), ri = 0.5f * rcp_est(g);
+    const float k = c2 ? -3.0f : (c1 ? -2.0f : -1.0f);
+    if constexpr (kStrict) {
+        // the adjoint divides by sums of t - psi_i, which carry the error of u:
+        // c in two parts (4.6e-15 of u off in the mean with one, 2.9e-15 with
+        // two; dL/ds of a 125x110x131 grid 3.5e-14 and 2.3e-14 off)
+        const dfl r = df_two_sum(ra, rb);
+        const float c = r.h * ri;
+        t = m + df_shift(u0, c, (fmaf(-2.0f * g, c, r.h) + fmaf(k * c, c, r.l)) * ri);
+    } else {
+        const float c = (ra + rb) * ri;
+        t = m + df_shift(u0, fmaf(k * c, c * ri, c));
+    }
+    if constexpr (kStrict) {
+        // m so large that t rounds to a value of the set
+        if (c1 && __double_as_longlong(t) <= __double_as_longlong(c2 ? v2 : v1))
+            return df_shifted_root<true>(m, v1, v2, v1 < 1e300 ? (v2 < 1e300 ? 3 : 2) : 1, q, t);
+    }
+    return c2 ? 3 : (c1 ? 2 : 1);
+}
+
 }  // namespace fmmgb

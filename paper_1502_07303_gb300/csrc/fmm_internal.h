@@ -61,25 +61,31 @@ struct Control {
     int error;
     int restart;                     // bound levels (restarts and raises)
     int host_restart;                // restarts the host enqueued (k_control)
-    // persistent march: ring queue positions and the count of bricks pushed
-    // and not yet marched, each on a line of its own (they are the only
-    // words every warp touches)
+    // one-launch schedules: the ready queue (bricks to march, first in first
+    // out), the waiting ring (bricks whose smallest work lies above the bound)
+    // and the count of bricks queued or marching, each on a line of its own
     alignas(128) unsigned long long q_head;
     alignas(128) unsigned long long q_tail;
+    unsigned long long w_tail;       // waiting ring: entries appended
     alignas(128) int pending;
     int pad2[31];
-    // continuous schedule: bound level (even = stable, odd = being raised),
-    // chunk counters of the scan for the current level, minima it saw
-    alignas(128) int epoch;
-    int scan_next;
-    int scan_done;
-    int scan_clean;                  // the last scan started with nothing in flight
-    int pad3;
-    unsigned long long scan_min[2];
-    unsigned long long wait_ns;      // limit of every device wait without progress
+    // the bound and the scan of the waiting ring that goes with it; a raise
+    // writes the other entry of level[] and then scan_word
+    alignas(128) unsigned long long scan_word;   // raise number << 32 | next chunk
+    unsigned long long w_head;       // waiting ring: entries below are scanned or being scanned
+    struct {
+        unsigned long long base, end;   // ring positions of the scan
+        int nchunks, chunk;
+        float bound;                    // marches start at or below it
+        int pad;
+    } level[2];
+    int scan_done;                   // chunks of the scan that are done
+    unsigned scan_min;               // smallest value it kept waiting (float bits)
+    int raise_lock;                  // raise number, one ahead while a raise is under way
     int hold;                        // testing: one brick counted as pending forever
-    int pad4[19];
+    unsigned long long wait_ns;      // limit of every device wait without progress
 };
+static_assert(sizeof(Control) == 640, "checkpoint images hold the control block");
 
 struct Geom {
     int nx, ny, nz;
@@ -140,17 +146,16 @@ constexpr int kSchedulePersistent = 2;
 constexpr int kScheduleContinuous = 3;
 constexpr int kScheduleCell = 4;     // cell-parallel bucketed march (fmm_cell.cu)
 constexpr int kMarchWarps = 4;   // bricks in flight per CTA of the march kernels
-#ifndef FMM_RAISE_DIV
-#define FMM_RAISE_DIV 2
-#endif
 // Continuous schedule: the bound rises once fewer bricks than this are queued
-// or marching (a fraction of the warps of the march launch).
-inline int raise_threshold(int march_ctas) { return march_ctas * kMarchWarps / FMM_RAISE_DIV; }
-// bricks one warp scans for the next bound (continuous schedule)
-#ifndef FMM_SCAN_CHUNK
-#define FMM_SCAN_CHUNK 1024
-#endif
-constexpr int kScanChunk = FMM_SCAN_CHUNK;
+// or marching: the warps of the march launch (half of them left 30% of the
+// 1024^3 march's warp time idle: 65 against 55 ms; twice as many: the same)
+inline int raise_threshold(int march_ctas) { return march_ctas * kMarchWarps; }
+// CTAs of a march launch: as many as fit, but no more warps than bricks
+inline int march_grid(int full, long long nbricks)
+{
+    const long long need = (nbricks + kMarchWarps - 1) / kMarchWarps;
+    return (int)(need < full ? (need > 0 ? need : 1) : full);
+}
 inline bool one_launch_schedule(int schedule)
 {
     return schedule == kSchedulePersistent || schedule == kScheduleContinuous;
@@ -191,15 +196,14 @@ struct DeviceState {
     void *bdelta;       // per-brick bucket width (h * min slowness / sqrt 3)
     uint8_t *tape;      // upwind set per cell or null
     void *bmin;         // 2 per brick: min |psi| of BAND cells per side
-    unsigned long long *fresh;   // 6 per brick: changed-halo masks (live)
-    unsigned long long *inmin;   // 2 per brick (sides -1, +1): smallest value a
-                                 // neighbour flagged in the masks since the
-                                 // brick last took them (bits of a double;
-                                 // all ones: none recorded)
+    unsigned long long *work;    // 1 per brick: smallest work it has, as float
+                                 // bits (rounded down; >= the bits of +inf:
+                                 // none), << 32 | flags (kWorkActive, kWorkWaiting)
+    unsigned long long *waiting; // waiting ring, laid out as the queue
     void *faces;        // deterministic mode, 6 x 64 per brick: its boundary
                         // layers (known value or +inf) as of the last pass
-    unsigned long long *inbox;   // 6 per brick: masks taken by the last selection
     unsigned int *dirty;         // 1 per brick: has pending overlap changes
+                                 // (phased schedule)
     int *list[2];       // work lists
     const int *nbr;     // 6 per brick: neighbour brick or -1 (batches only)
     unsigned long long *queue;   // persistent march: ring of (seq << 32 | brick + 1)

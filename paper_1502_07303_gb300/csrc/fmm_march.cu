@@ -8,28 +8,22 @@
 //   Initialize_Heap_Parallel (Alg. 9)       -> k_march<mode 0> (one relax of
 //                                               every cell next to a FIX cell)
 //   local minima + AllReduce (Alg. 16)      -> k_reduce + k_control
-//   March_Narrow_Band_Parallel (Alg. 12)    -> march_brick, run by one of three
-//                                               restart schedules (below)
-//   Collect/Exchange/Integrate (Alg. 13-15) -> write-back to HBM plus per-face
-//                                               "fresh" bit masks on the
-//                                               neighbour brick, whose next
-//                                               staging reads the new values
+//   March_Narrow_Band_Parallel (Alg. 12)    -> sweep_brick (fmm_sweep.cuh), run
+//                                               by one of three restart
+//                                               schedules (below)
+//   Collect/Exchange/Integrate (Alg. 13-15) -> write-back to HBM plus the
+//                                               smallest changed value and the
+//                                               changed face in the neighbour's
+//                                               work word; its next staging
+//                                               reads the new values
 //   second march of Alg. 16                 -> the neighbour is marched again
 //                                               (queued, or listed as dirty)
 //
-// Restart schedules: continuous (k_march_continuous: one launch for the whole
+// Restart schedules: continuous (k_march_queue: one launch for the whole
 // solve, bricks from a device-side queue, the bound raised in the kernel when
-// a restart runs out of parallel work), persistent (k_seed +
-// k_march_persistent: one queue-driven launch per restart) and phased
-// (k_select + k_march<mode 1>: one launch per pass over a work list).
-//
-// Inside a brick (one warp per brick) the heap of Algorithm 12 is replaced by
-// a bucketed, label-correcting march: each round accepts every BAND cell whose |psi| is
-// within a bucket width of the brick's BAND minimum (and within the restart
-// bound), then every cell next to a newly accepted cell re-solves Algorithm
-// 11.  A cell whose value drops is reset to BAND even if it was accepted,
-// exactly as Algorithm 10 resets KNOWN_NEW/KNOWN_OLD points, so the march
-// ends at the same local fixed point as the heap march.
+// a restart runs out of parallel work), persistent (k_seed + k_march_queue with
+// a fixed bound: one launch per restart) and phased (k_select + k_march<mode
+// 1>: one launch per pass over a work list).
 //
 // A brick never solves cells it does not own: halo cells are read-only
 // upwind data.  Every cell therefore has a single writer, and values only
@@ -38,9 +32,7 @@
 // marched again before termination can be declared.
 #include "fmm_internal.h"
 #include "fmm_queue.cuh"
-#include "fmm_fp64.cuh"
-#include "fmm_df.cuh"
-#include "fmm_lanes.cuh"
+#include "fmm_sweep.cuh"
 
 #include <cfloat>
 #include <cmath>
@@ -50,14 +42,6 @@
 namespace fmmgb {
 namespace {
 
-template <typename real>
-__device__ __forceinline__ real inf_v();
-template <>
-__device__ __forceinline__ float inf_v<float>() { return __int_as_float(0x7f800000); }
-template <>
-__device__ __forceinline__ double inf_v<double>() { return __longlong_as_double(0x7ff0000000000000ll); }
-
-__device__ __forceinline__ bool is_known(uint8_t tg) { return (tg & ST_MASK) >= ST_KNOWN; }
 
 __device__ __forceinline__ void brick_coords(const Geom &g, long long b, int &bx, int &by,
                                              int &bz)
@@ -85,291 +69,6 @@ __device__ __forceinline__ long long neighbour_brick(const Geom &g, const int *n
     if (nbx < 0 || nbx >= g.nbx || nby < 0 || nby >= g.nby || nbz < 0 || nbz >= g.nbz)
         return -1;
     return ((long long)nbz * g.nby + nby) * g.nbx + nbx;
-}
-
-// ---------------------------------------------------------------------------
-// Algorithm 11 (Solve_Quadratic_Parallel) on a staged tile.
-//
-// kv holds the value of every KNOWN/FIX cell of the brick and its halo, +inf
-// for an unknown halo cell and the marked (sign bit set) value of every other
-// brick cell, so "G in KNOWN and |psi_n| < |psi_cell|" is "kv_n < Tc" on the
-// unsigned bit patterns (klt).
-// The per-axis choice and the nested upwind sets (each time dropping the
-// largest psi_i) follow the algorithm.  Algorithm 11 keeps the smallest
-// causal root over the sets; going from the full set down, the first causal
-// root already is that minimum: a causal root t_S of a nested set S satisfies
-// sum over all axes of max(t_S - psi_i, 0)^2 >= (h/F)^2, so t_S is never
-// below the unique solution t* of sum max(t - psi_i, 0)^2 = (h/F)^2, and t*
-// is the causal root of the set {i : psi_i < t*}.  The loop therefore stops
-// at the first causal root.  set_out receives its upwind set (2 bits per
-// axis: 1 = minus, 2 = plus neighbour).
-//
-// |psi| values are never negative, so double comparisons are done on the
-// bit patterns (integer compares keep them off the FP64 pipe).
-// ---------------------------------------------------------------------------
-
-__device__ __forceinline__ bool lt(double a, double b)
-{
-    // valid for values >= 0 and +inf; a negative discriminant has the sign
-    // bit set and compares below every non-negative value
-    return __double_as_longlong(a) < __double_as_longlong(b);
-}
-__device__ __forceinline__ bool lt(float a, float b) { return a < b; }
-__device__ __forceinline__ double vmin(double a, double b) { return lt(a, b) ? a : b; }
-__device__ __forceinline__ float vmin(float a, float b) { return fminf(a, b); }
-
-// Tile entries of the march: a known value as it is, any other brick cell
-// with its sign bit set (the "not known" mark, see WarpTile).  Compared as
-// unsigned bit patterns, a marked entry orders above every value including
-// +inf, so the smaller of two neighbours is the known one and a marked
-// entry is never below a cell's value: Algorithm 11's "known and smaller"
-// test costs no decoding.
-__device__ __forceinline__ bool klt(double a, double b)
-{
-    return (unsigned long long)__double_as_longlong(a) < (unsigned long long)__double_as_longlong(b);
-}
-__device__ __forceinline__ bool klt(float a, float b) { return __float_as_uint(a) < __float_as_uint(b); }
-__device__ __forceinline__ double kmin(double a, double b) { return klt(a, b) ? a : b; }
-__device__ __forceinline__ float kmin(float a, float b)
-{
-    return __uint_as_float(umin(__float_as_uint(a), __float_as_uint(b)));
-}
-// mark / unmark (set / clear the sign bit, on the high word of a double)
-__device__ __forceinline__ double kmark(double v)
-{
-    return __hiloint2double(__double2hiint(v) | (int)0x80000000, __double2loint(v));
-}
-__device__ __forceinline__ float kmark(float v) { return __uint_as_float(__float_as_uint(v) | 0x80000000u); }
-__device__ __forceinline__ double kval(double v)
-{
-    return __hiloint2double(__double2hiint(v) & 0x7fffffff, __double2loint(v));
-}
-__device__ __forceinline__ float kval(float v) { return __uint_as_float(__float_as_uint(v) & 0x7fffffffu); }
-
-// Double square root without the FP64 pipe's slow conversions (fmm_fp64.cuh).
-__device__ __forceinline__ double vsqrt(double v) { return sqrt_fp64(v); }
-// Single precision: x * rsqrt(x) (a few ulp, far below the fp32 tolerance;
-// 0 stays 0).  The +inf speed term of an obstacle cell gives NaN, which fails
-// every causality test of Algorithm 11, so the cell's candidate is +inf.
-__device__ __forceinline__ float vsqrt(float v) { return v * rsqrtf(fmaxf(v, 1e-37f)); }
-
-// The quadratic of Algorithm 11, sum_i (t - psi_i)^2 / h^2 = 1/F^2 over the
-// upwind set, is solved for the unknown shifted by the smallest upwind value
-// m: t = m + u, delta_i = psi_i - m, sum_i (u - delta_i)^2 = q with
-// q = (h/F)^2.  The coefficients stay of order h, so rounding does not grow
-// with psi (in psi itself b^2 and 4ac would cancel to ~3 (psi F/h)^2 ulp).
-// The causality test psi_i < t is delta_i < u; the kernels that record the
-// upwind sets for the adjoint make it on t = m + u and the values the cells
-// hold (on rounded shifts delta_i < u can hold while t rounds to psi_i, and a
-// recorded set must point strictly downhill).  q is the cell's speed term.
-//
-// Per axis the upwind value is the smaller known neighbour if it is below
-// Tc; with a tape (kTape) the side it came from is kept as well (the minus
-// side on a tie; without a tape the compiler drops the sides).  The per-axis values are sorted once (a stable sort, so
-// equal values keep the lower axis first and the higher axis is dropped
-// first).  The smallest has delta = 0, so only the other two enter
-// S = sum delta_i and Q = sum delta_i^2 (a dropped axis contributes 0):
-// disc = S^2 - k (Q - q), u = (S + sqrt(disc)) / k, causal when the largest
-// remaining delta is below u (with a tape: when t = m + u exceeds the largest
-// remaining value).  All lanes of a warp evaluate their full set
-// together; a lane whose full set is not causal (about 1% of solves) goes
-// round the loop again.
-template <typename real>
-__device__ __forceinline__ void cswap(real &a, unsigned &ca, real &b, unsigned &cb)
-{
-    if (lt(b, a)) {
-        const real t = a;
-        a = b;
-        b = t;
-        const unsigned c = ca;
-        ca = cb;
-        cb = c;
-    }
-}
-
-template <typename real, bool kTape>
-__device__ __forceinline__ real solve_cell(const real *kv, int ti, real Tc, real q,
-                                           uint8_t &set_out)
-{
-    const int off[3] = {1, kTile, kTile * kTile};
-    const real INF = inf_v<real>();
-    real v[3];
-    unsigned code[3];
-    int nd = 0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const real vm = kv[ti - off[a]], vp = kv[ti + off[a]];
-        const real w = kmin(vm, vp);
-        const bool up = klt(w, Tc);
-        v[a] = up ? w : INF;
-        code[a] = up ? (klt(vp, vm) ? 2u : 1u) << (2 * a) : 0u;   // dead without a tape
-        nd += up;
-    }
-    set_out = 0;
-    if (nd == 0)
-        return INF;
-    if constexpr (!kTape && sizeof(real) == 4) {
-        // without sides to carry along: a min / max network
-        const float a = fminf(v[0], v[1]), b = fmaxf(v[0], v[1]);
-        const float d = fminf(b, v[2]);
-        v[2] = fmaxf(b, v[2]);
-        v[0] = fminf(a, d);
-        v[1] = fmaxf(a, d);
-    } else {
-        // stable sort of three (adjacent compare-exchange, strict less-than)
-        cswap(v[0], code[0], v[1], code[1]);
-        cswap(v[1], code[1], v[2], code[2]);
-        cswap(v[0], code[0], v[1], code[1]);
-    }
-    const real m = v[0];
-    if constexpr (sizeof(real) == 8) {
-        // double grids: the root in double-float arithmetic (fmm_df.cuh),
-        // unless the speed term is outside its range (an obstacle's +inf)
-        if (in_float_range(q)) {
-            double t = 0.0;
-            const int k = df_shifted_root<kTape>(v[0], v[1], v[2], nd, q, t);
-            if (k == 0)
-                return INF;
-            set_out = (uint8_t)(code[0] | (k >= 2 ? code[1] : 0u) | (k == 3 ? code[2] : 0u));
-            return t;
-        }
-    }
-    real d1 = nd >= 2 ? v[1] - m : (real)0;
-    real d2 = nd >= 3 ? v[2] - m : (real)0;
-#pragma unroll 1
-    for (; nd != 0; --nd) {
-        const real S = d1 + d2;
-        const real Q = fma(d2, d2, d1 * d1);
-        const real k = nd == 3 ? (real)3 : (nd == 2 ? (real)2 : (real)1);
-        const real disc = fma(-k, Q - q, S * S);
-        if (!lt(disc, (real)0)) {
-            const real inv_k = nd == 3 ? (real)(1.0 / 3.0) : (nd == 2 ? (real)0.5 : (real)1);
-            const real u = (S + vsqrt(disc)) * inv_k;
-            // causal: the largest remaining delta is below u; with a tape,
-            // the root above the largest value as the cells hold it (the
-            // upwind sets recorded for the adjoint must point strictly
-            // downhill); one value: u > 0
-            const real t = m + u;
-            const bool causal = kTape ? (nd == 1 ? lt((real)0, u) : lt(nd == 3 ? v[2] : v[1], t))
-                                      : lt(nd == 3 ? d2 : d1, u);
-            if (causal) {
-                set_out = (uint8_t)(code[0] | (nd >= 2 ? code[1] : 0u) | (nd == 3 ? code[2] : 0u));
-                return t;
-            }
-        }
-        // drop the largest remaining value
-        if (nd == 3)
-            d2 = (real)0;
-        else
-            d1 = (real)0;
-    }
-    return INF;
-}
-
-// Algorithm 11 with cells of size h * hy * hz: h_i^2 (t - psi_i)^2 summed
-// over the set equals F^-2, i.e. sum_i w_i (u - delta_i)^2 = q with
-// w_i = (h / h_i)^2 (w_x = 1), q = (h/F)^2 and the same shift t = m + u.
-// The per-axis values are sorted together with their weights (and sides);
-// with K = sum w_i, S = sum w_i delta_i and Q = sum w_i delta_i^2 over the
-// set, disc = S^2 - K (Q - q), evaluated as K q - sum_{i<j} w_i w_j
-// (delta_i - delta_j)^2, and u = (S + sqrt(disc)) / K; the largest remaining
-// value is dropped while the set is not causal, as above.
-template <typename real>
-__device__ __forceinline__ void cswap_w(real &a, real &wa, unsigned &ca, real &b, real &wb, unsigned &cb)
-{
-    if (lt(b, a)) {
-        const real t = a, tw = wa;
-        a = b;
-        b = t;
-        wa = wb;
-        wb = tw;
-        const unsigned c = ca;
-        ca = cb;
-        cb = c;
-    }
-}
-__device__ __forceinline__ float vdiv(float a, float b) { return a / b; }
-__device__ __forceinline__ double vdiv(double a, double b) { return div_fp64(a, b); }
-
-template <typename real, bool kTape>
-__device__ __forceinline__ real solve_cell_w(const real *kv, int ti, real Tc, real q, real wy,
-                                             real wz, uint8_t &set_out)
-{
-    const int off[3] = {1, kTile, kTile * kTile};
-    const real wax[3] = {(real)1, wy, wz};
-    const real INF = inf_v<real>();
-    real v[3], w[3];
-    unsigned code[3];
-    int nd = 0;
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-        const real vm = kv[ti - off[a]], vp = kv[ti + off[a]];
-        const real mn = kmin(vm, vp);
-        const bool up = klt(mn, Tc);
-        v[a] = up ? mn : INF;
-        w[a] = up ? wax[a] : (real)0;
-        code[a] = up ? (klt(vp, vm) ? 2u : 1u) << (2 * a) : 0u;   // dead without a tape
-        nd += up;
-    }
-    set_out = 0;
-    if (nd == 0)
-        return INF;
-    // stable sort of three, each weight and side with its value
-    cswap_w(v[0], w[0], code[0], v[1], w[1], code[1]);
-    cswap_w(v[1], w[1], code[1], v[2], w[2], code[2]);
-    cswap_w(v[0], w[0], code[0], v[1], w[1], code[1]);
-    const real m = v[0];
-    real d1 = nd >= 2 ? v[1] - m : (real)0;
-    real d2 = nd >= 3 ? v[2] - m : (real)0;
-    const real w0 = w[0];
-    real w1 = nd >= 2 ? w[1] : (real)0;
-    real w2 = nd >= 3 ? w[2] : (real)0;
-#pragma unroll 1
-    for (; nd != 0; --nd) {
-        const real K = w0 + w1 + w2;
-        const real S = fma(w1, d1, w2 * d2);
-        // S^2 - K (Q - q) = K q - sum_{i<j} w_i w_j (delta_i - delta_j)^2
-        // (Lagrange's identity): with unequal weights S^2 and K Q nearly
-        // cancel, the pairwise form does not
-        const real e = d1 - d2;
-        const real P = fma(w0 * w1, d1 * d1, fma(w0 * w2, d2 * d2, (w1 * w2) * (e * e)));
-        const real disc = fma(K, q, -P);
-        if (!lt(disc, (real)0)) {
-            const real u = vdiv(S + vsqrt(disc), K);
-            const real t = m + u;   // causal as in solve_cell
-            const bool causal = kTape ? (nd == 1 ? lt((real)0, u) : lt(nd == 3 ? v[2] : v[1], t))
-                                      : lt(nd == 3 ? d2 : d1, u);
-            if (causal) {
-                set_out = (uint8_t)(code[0] | (nd >= 2 ? code[1] : 0u) | (nd == 3 ? code[2] : 0u));
-                return t;
-            }
-        }
-        // drop the largest remaining value with its weight
-        if (nd == 3) {
-            d2 = (real)0;
-            w2 = (real)0;
-        } else {
-            d1 = (real)0;
-            w1 = (real)0;
-        }
-    }
-    return INF;
-}
-
-// Warp minimum of non-negative values (or +inf): their bit patterns order
-// like the values, so the integer reductions of the warp do it exactly (a
-// double in two steps, high word then low word).
-__device__ __forceinline__ float warp_min(float v)
-{
-    return __uint_as_float(__reduce_min_sync(0xffffffffu, __float_as_uint(v)));
-}
-__device__ __forceinline__ double warp_min(double v)
-{
-    const unsigned long long b = (unsigned long long)__double_as_longlong(v);
-    const unsigned hi = __reduce_min_sync(0xffffffffu, (unsigned)(b >> 32));
-    const unsigned lo =
-        __reduce_min_sync(0xffffffffu, (unsigned)(b >> 32) == hi ? (unsigned)b : 0xffffffffu);
-    return __longlong_as_double((long long)(((unsigned long long)hi << 32) | lo));
 }
 
 // ---------------------------------------------------------------------------
@@ -623,17 +322,12 @@ __global__ void __launch_bounds__(kThreads) k_load_speed(Geom g, double h, doubl
 }
 
 // ---------------------------------------------------------------------------
-// The brick march: one warp per brick.  kMode 0: Algorithm 9 over all bricks
-// (every non-FIX cell next to a known cell is solved once, nothing is
-// accepted).  kMode 1: Algorithm 12 up to the restart bound over the bricks
-// of work list `which`.
-//
-// Lane l owns the 16 cells c = l + 32 k (k = 0..15) of the brick: x = l % 8,
-// y = (l / 8) % 4 + 4 (k % 2), z = k / 2.  Cell sets (BAND, KNOWN, frozen,
-// side, accepted, to-solve) are 16-bit masks per lane, bit k for cell
-// l + 32 k, so the per-round passes touch only the cells in a set.  The cells
-// to solve in a round are compacted into a list by a warp prefix sum, so all
-// 32 lanes solve.
+// The brick march (fmm_sweep.cuh): one warp per brick, four bricks per CTA.  It
+// is bound by the length of a brick's chain of steps where a grid has few
+// bricks per warp, and by the ALU (float) and FP64 (double) pipes where it has
+// many.  256^3 level set of 32 spheres, whole call: 1.8 ms in float, 4.9 ms in
+// double (5.7 and 12.0 ms with the bucketed march this replaced); 1024^3 sphere
+// in double 59 ms (236 ms).
 // ---------------------------------------------------------------------------
 
 #ifndef FMM_MARCH_BLOCKS_F32
@@ -646,489 +340,20 @@ __global__ void __launch_bounds__(kThreads) k_load_speed(Geom g, double h, doubl
 #define FMM_MARCH_BLOCKS_F64_TAPE 5
 #endif
 // Resident CTAs per SM the march kernels are compiled for (registers); the
-// warp tiles (5.1 / 5.6 KB in float, 9.0 / 9.5 KB in double, without / with
-// the tape) allow these as well.  Measured on the 1024^3 sphere: fp64 with
-// 4 / 5 / 6 CTAs 261 / 236 / 242 ms (six leave 80 registers and spill),
-// fp32 with 6 / 7 / 8 CTAs 122 / 115 / 115 ms (eight slow the 256^3 case).
+// warp tiles (5.7 / 6.2 KB in float, 9.7 / 10.2 KB in double, without / with
+// the tape) allow these as well.  Six fp64 CTAs would leave 80 registers and
+// spill.
 template <typename real, bool kTape>
 constexpr int march_min_blocks()
 {
     return sizeof(real) == 4 ? FMM_MARCH_BLOCKS_F32 : (kTape ? FMM_MARCH_BLOCKS_F64_TAPE : FMM_MARCH_BLOCKS_F64);
 }
-constexpr unsigned FULL = 0xffffffffu;
-
-// The brick and its face halo in one 10^3 tile (x fastest), shifted by one
-// entry so that every row of 8 brick cells starts on a 16-byte boundary in
-// double and an 8-byte boundary in float: kMT0 is the tile index of brick
-// cell (0, 0, 0), kMH0 that of halo position (0, 0, 0).  A brick cell holds
-// its current |psi|, with the sign bit set unless the cell is KNOWN or FIX; a
-// halo cell holds the neighbour's known value or +inf.  One array for the
-// known values and the current values keeps the fp64 tile at 9.5 KB a warp,
-// which lets five CTAs of four warps share an SM.
-constexpr int kMH0 = 1;
-constexpr int kMT0 = kMH0 + 1 + kTile + kTile * kTile;
-constexpr int kMTile = kMH0 + kTile3 + 1;
-
-__device__ __forceinline__ int mt_of(int c)
-{
-    return kMT0 + (c & 7) + kTile * ((c >> 3) & 7) + kTile * kTile * (c >> 6);
-}
-
+// Shared memory of a march CTA.
 template <typename real, bool kTape>
-struct WarpTile {
-    alignas(16) real kv[kMTile];       // brick (marked unless known) and face halo
-    alignas(16) uint8_t tp[kTape ? kB3 : 16];   // upwind sets (with a tape)
-    alignas(16) uint16_t list[kB3];    // compacted cells to solve (the tags
-                                       // while staging and writing back)
-    unsigned improved[32]; // per owner lane: cells whose value dropped
+struct MarchSmem {
+    WarpTile<real, kTape> tile[kMarchWarps];
+    int order[(kSweepSteps + 1) * 32];
 };
-static_assert(sizeof(WarpTile<float, false>) % 16 == 0 && sizeof(WarpTile<double, false>) % 16 == 0 &&
-                  sizeof(WarpTile<float, true>) % 16 == 0 && sizeof(WarpTile<double, true>) % 16 == 0,
-              "every warp's tile starts on a 16-byte boundary");
-static_assert((kMT0 * 8) % 16 == 0 && (kTile * 8) % 16 == 0 && (kMT0 * 4) % 8 == 0 && (kTile * 4) % 8 == 0,
-              "brick rows of the tile start on 16 (double) / 8 (float) byte boundaries");
-
-// The q-th 16 bytes of a brick in brick order (cells c = x + 8 y + 64 z) to
-// and from the tile rows: two cells per 16 bytes in double (four per row),
-// four in float (two per row, stored as two 8-byte halves).  row_load clears
-// the marks: the brick in global memory holds |psi|.
-__device__ __forceinline__ void row_store(double *kv, int q, uint4 x)
-{
-    const int row = q >> 2;   // y + 8 z
-    reinterpret_cast<uint4 *>(kv + kMT0 + kTile * (row & 7) + kTile * kTile * (row >> 3))[q & 3] = x;
-}
-__device__ __forceinline__ void row_store(float *kv, int q, uint4 x)
-{
-    const int row = q >> 1;
-    uint2 *d = reinterpret_cast<uint2 *>(kv + kMT0 + kTile * (row & 7) + kTile * kTile * (row >> 3) + 4 * (q & 1));
-    d[0] = make_uint2(x.x, x.y);
-    d[1] = make_uint2(x.z, x.w);
-}
-__device__ __forceinline__ uint4 row_load(const double *kv, int q)
-{
-    const int row = q >> 2;
-    uint4 x = reinterpret_cast<const uint4 *>(kv + kMT0 + kTile * (row & 7) + kTile * kTile * (row >> 3))[q & 3];
-    x.y &= 0x7fffffffu;   // high words
-    x.w &= 0x7fffffffu;
-    return x;
-}
-__device__ __forceinline__ uint4 row_load(const float *kv, int q)
-{
-    const int row = q >> 1;
-    const uint2 *d =
-        reinterpret_cast<const uint2 *>(kv + kMT0 + kTile * (row & 7) + kTile * kTile * (row >> 3) + 4 * (q & 1));
-    const uint2 a = d[0], b = d[1];
-    return make_uint4(a.x & 0x7fffffffu, a.y & 0x7fffffffu, b.x & 0x7fffffffu, b.y & 0x7fffffffu);
-}
-
-// Cells of lane l next to a halo cell flagged in the per-face masks F[6]
-// (face bit = u + 8 v with (u, v) the two in-face coordinates).
-__device__ __forceinline__ unsigned face_mask(const unsigned long long F[kFaces], int lane)
-{
-    const int x = lane & 7, r = (lane >> 3) & 3;
-    unsigned n = 0;
-#pragma unroll 4
-    for (int k = 0; k < 16; ++k) {
-        const int y = r + 4 * (k & 1), z = k >> 1;
-        bool hit = false;
-        if (x == 0)
-            hit = hit || ((F[0] >> (y + 8 * z)) & 1ull);
-        if (x == 7)
-            hit = hit || ((F[1] >> (y + 8 * z)) & 1ull);
-        if (y == 0)
-            hit = hit || ((F[2] >> (x + 8 * z)) & 1ull);
-        if (y == 7)
-            hit = hit || ((F[3] >> (x + 8 * z)) & 1ull);
-        if (z == 0)
-            hit = hit || ((F[4] >> (x + 8 * y)) & 1ull);
-        if (z == 7)
-            hit = hit || ((F[5] >> (x + 8 * y)) & 1ull);
-        if (hit)
-            n |= 1u << k;
-    }
-    return n;
-}
-
-struct MarchStats {
-    unsigned long long marches, rounds, accepted, exchanges, solves;
-};
-
-// One brick march.  F_in: the halo cells whose known value changed since the
-// brick last ran (kMode 1); kMode 0 derives them from the known halo cells.
-// kFresh: read the brick and halo through L2 (the persistent kernel, where the
-// brick may have been written by another SM during the same launch).  kTape:
-// record the upwind set of every solve for the adjoint (without it the
-// compiler drops the set bookkeeping of Algorithm 11 altogether).  kAniso:
-// cells of unequal sizes (the weighted solve).  On
-// return, lanes 0..5 hold in notify_m / notify_nb the changed boundary cells
-// and the neighbour brick across face = lane (mode 1), and every lane holds in
-// notify_v[2] the smallest flagged value of each side (+inf: none).
-template <typename real, bool kHetero, int kMode, bool kFresh, bool kTape, bool kAniso>
-__device__ __forceinline__ void march_brick(const Geom &g, const DeviceState &s, const SolveParams &p,
-                                            double spd_const_term, WarpTile<real, kTape> &W, long long b,
-                                            const unsigned long long *F_in, real bound0, real bound1,
-                                            int lane, unsigned long long &notify_m,
-                                            long long &notify_nb, real *notify_v, MarchStats &st)
-{
-    real *T = (real *)s.T;
-    uint8_t *tag = s.tag;
-    const real *spd = (const real *)s.spd;
-    const real *bdelta = (const real *)s.bdelta;
-    real *bmin = (real *)s.bmin;
-    const real INF = inf_v<real>();
-    const int lx = lane & 7, lr = (lane >> 3) & 3;
-    const int tb = kMT0 + lx + kTile * lr;   // tile index of the lane's cell k = 0
-    long long nbi[kFaces];
-#pragma unroll
-    for (int f = 0; f < kFaces; ++f)
-        nbi[f] = neighbour_brick(g, s.nbr, b, f);
-    const long long base = b * kB3;
-
-    // ---- stage the brick ---------------------------------------------------
-    // The brick's values, tags (and tape) are contiguous: 16-byte loads copy
-    // them into shared memory (the values into the rows of the tile, the tags
-    // into the list buffer, unused until the rounds), then every lane marks
-    // its own cells there.
-    uint8_t *const stag = reinterpret_cast<uint8_t *>(W.list);
-    {
-        constexpr int kVecs = kB3 * (int)sizeof(real) / 16 / 32;   // 16-byte loads per lane
-        const uint4 *gv = reinterpret_cast<const uint4 *>(T + base);
-#pragma unroll
-        for (int j = 0; j < kVecs; ++j) {
-            const int q = lane + 32 * j;
-            const uint4 x = kFresh ? __ldcg(gv + q) : gv[q];
-            row_store(W.kv, q, x);
-        }
-        const uint4 *gt = reinterpret_cast<const uint4 *>(tag + base);
-        reinterpret_cast<uint4 *>(stag)[lane] = kFresh ? __ldcg(gt + lane) : gt[lane];
-        if (kTape) {
-            const uint4 *gp = reinterpret_cast<const uint4 *>(s.tape + base);
-            reinterpret_cast<uint4 *>(W.tp)[lane] = kFresh ? __ldcg(gp + lane) : gp[lane];
-        }
-    }
-    __syncwarp();
-    unsigned band = 0, known = 0, fix = 0, out = 0, neg = 0;
-    real r0 = INF, r1 = INF;   // lane minimum of the BAND cells of each side
-#pragma unroll 4
-    for (int k = 0; k < 16; ++k) {
-        const int c = lane + 32 * k;
-        const int ti = tb + 40 * (k & 1) + 100 * (k >> 1);
-        const real v = W.kv[ti];
-        const uint8_t t = stag[c];
-        const uint8_t sv = t & ST_MASK;
-        if (sv < ST_KNOWN)
-            W.kv[ti] = kmark(v);
-        band |= (unsigned)(sv == ST_BAND) << k;
-        known |= (unsigned)(sv >= ST_KNOWN) << k;
-        fix |= (unsigned)(sv == ST_FIX) << k;
-        out |= (unsigned)((t & TG_OUT) != 0) << k;
-        neg |= (unsigned)((t & TG_NEG) != 0) << k;
-        if (sv == ST_BAND) {
-            if (t & TG_NEG)
-                r0 = vmin(r0, v);
-            else
-                r1 = vmin(r1, v);
-        }
-    }
-    W.improved[lane] = 0u;
-    const unsigned frozen = fix | out;
-    // ---- halo: the face layers of the six neighbours (read-only) ----------
-    unsigned long long F[kFaces];
-#pragma unroll
-    for (int f = 0; f < kFaces; ++f)
-        F[f] = kMode == 0 ? 0ull : F_in[f];
-#pragma unroll
-    for (int f = 0; f < kFaces; ++f) {
-        const long long nb = nbi[f];
-        const int axis = f >> 1, dir = (f & 1) ? 1 : -1;
-#pragma unroll
-        for (int half = 0; half < 2; ++half) {
-            const int q = lane + 32 * half, u = q & 7, v = q >> 3;
-            real val = INF;
-            if (kMode == 1 && nb >= 0 && s.faces) {
-                // deterministic mode: the neighbour's layer as of the last pass
-                val = __ldcg((const real *)s.faces + nb * (kFaces * 64) + (f ^ 1) * 64 + q);
-            } else if (nb >= 0) {
-                const int edge = dir < 0 ? kB - 1 : 0;
-                const int cx = axis == 0 ? edge : u;
-                const int cy = axis == 1 ? edge : (axis == 0 ? u : v);
-                const int cz = axis == 2 ? edge : v;
-                const long long ci = nb * kB3 + cx + kB * cy + kB * kB * cz;
-                const uint8_t ntg = __ldcg(tag + ci);
-                const real nv = __ldcg(T + ci);
-                if (is_known(ntg))
-                    val = nv;
-            }
-            const int hedge = dir < 0 ? 0 : kTile - 1;
-            const int hx = axis == 0 ? hedge : u + 1;
-            const int hy = axis == 1 ? hedge : (axis == 0 ? u + 1 : v + 1);
-            const int hz = axis == 2 ? hedge : v + 1;
-            W.kv[kMH0 + hx + kTile * hy + kTile * kTile * hz] = val;
-            if (kMode == 0) {
-                // Algorithm 9: every known halo cell updates its neighbours
-                const unsigned bal = __ballot_sync(FULL, lt(val, INF));
-                F[f] |= (unsigned long long)bal << (32 * half);
-            }
-        }
-    }
-    __syncwarp();
-
-    unsigned relax = face_mask(F, lane);
-    if (kMode == 0)
-        relax |= neighbour_mask(known, lane);
-    relax &= ~frozen;
-
-    const real delta = (real)p.bucket * bdelta[b];
-    unsigned acc_any = 0;
-    int rounds = 0;
-    real m0 = INF, m1 = INF;
-    // Settled cells: KNOWN cells at or below the band minimum of their side.
-    // An accepted value is at least the band minimum of its round, and an
-    // update from an upwind value v never goes below v, so while the minimum
-    // does not fall no later acceptance can lower a settled cell and the
-    // cell is left out of the solves.  The minimum normally only rises (a
-    // value computed from an accepted neighbour v is a causal root above v),
-    // but a halo value staged before its change flag arrived (written by a
-    // neighbour brick during this march) can let a relaxed cell drop below it;
-    // when the minimum of a side falls, that side's settled cells are
-    // released.  pend: cells accepted at or below the largest lim so far
-    // (pl0, pl1) that settle once the minimum of their side reaches it.
-    unsigned settled = 0, pend = 0;
-    real pl0 = (real)0, pl1 = (real)0;
-    real mp0 = (real)0, mp1 = (real)0;   // band minima of the previous round
-    for (;;) {
-        // compact the cells to solve (warp prefix sum of the lane counts)
-        const int cnt = __popc(relax);
-        int pre = cnt;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int t = __shfl_up_sync(FULL, pre, o);
-            if (lane >= o)
-                pre += t;
-        }
-        const int n_items = __shfl_sync(FULL, pre, 31);
-        pre -= cnt;
-        st.solves += (unsigned long long)n_items;
-        for (unsigned m = relax; m; m &= m - 1u)
-            W.list[pre++] = (uint16_t)(lane + 32 * (__ffs(m) - 1));
-        __syncwarp();
-        // Algorithm 10/11: solve, then apply (Jacobi within 32 cells)
-        for (int i0 = 0; i0 < n_items; i0 += 32) {
-            const int i = i0 + lane;
-            int c = -1, ti = 0;
-            real cand = INF, tc = INF;
-            uint8_t cset = 0;
-            if (i < n_items) {
-                c = W.list[i];
-                ti = mt_of(c);
-                tc = kval(W.kv[ti]);
-                const real sp = kHetero ? __ldg(spd + base + c) : (real)spd_const_term;
-                if constexpr (kAniso)
-                    cand = solve_cell_w<real, kTape>(W.kv, ti, tc, sp, (real)p.wy, (real)p.wz, cset);
-                else
-                    cand = solve_cell<real, kTape>(W.kv, ti, tc, sp, cset);
-            }
-            __syncwarp();
-            // each cell appears once in the list, so tc is still its value
-            if (c >= 0 && lt(cand, tc)) {
-                W.kv[ti] = kmark(cand);
-                if (kTape)
-                    W.tp[c] = cset;
-                atomicOr(&W.improved[c & 31], 1u << (c >> 5));
-            }
-            __syncwarp();
-        }
-        // a cell whose value dropped is BAND again (Algorithm 10)
-        const unsigned imp = W.improved[lane];
-        W.improved[lane] = 0u;
-        band |= imp;
-        known &= ~imp;
-        settled &= ~imp;
-        pend &= ~imp;
-        // minimum of the BAND cells of each side (the heap tops): the cells
-        // the last accept scan left plus the cells that just dropped
-        real l0 = r0, l1 = r1;
-        for (unsigned m = imp; m; m &= m - 1u) {
-            const int k = __ffs(m) - 1;
-            const real v = kval(W.kv[tb + 40 * (k & 1) + 100 * (k >> 1)]);
-            if ((neg >> k) & 1u)
-                l0 = vmin(l0, v);
-            else
-                l1 = vmin(l1, v);
-        }
-        m0 = warp_min(l0);
-        m1 = warp_min(l1);
-        if (kMode == 0)
-            break;
-        if (lt(m0, mp0))
-            settled &= ~neg;
-        if (lt(m1, mp1))
-            settled &= neg;
-        mp0 = m0;
-        mp1 = m1;
-        if (rounds == 0) {
-            // cells that were KNOWN when the march began
-            for (unsigned m = known & ~settled; m; m &= m - 1u) {
-                const int k = __ffs(m) - 1;
-                if (!lt((neg >> k) & 1u ? m0 : m1, W.kv[tb + 40 * (k & 1) + 100 * (k >> 1)]))
-                    settled |= 1u << k;
-            }
-        }
-        if (!lt(m0, pl0)) {
-            settled |= pend & neg;
-            pend &= ~neg;
-        }
-        if (!lt(m1, pl1)) {
-            settled |= pend & ~neg;
-            pend &= neg;
-        }
-        // accept the lowest bucket up to the restart bound; the rest give
-        // the band minimum of the next round
-        const real lim0 = vmin(m0 + delta, bound0), lim1 = vmin(m1 + delta, bound1);
-        unsigned acc = 0;
-        r0 = INF;
-        r1 = INF;
-        for (unsigned m = band; m; m &= m - 1u) {
-            const int k = __ffs(m) - 1;
-            const int ti = tb + 40 * (k & 1) + 100 * (k >> 1);
-            const real v = kval(W.kv[ti]);
-            const bool ng = (neg >> k) & 1u;
-            if (!lt(ng ? lim0 : lim1, v)) {
-                acc |= 1u << k;
-                W.kv[ti] = v;
-            } else if (ng) {
-                r0 = vmin(r0, v);
-            } else {
-                r1 = vmin(r1, v);
-            }
-        }
-        band &= ~acc;
-        known |= acc;
-        const int nacc = __reduce_add_sync(FULL, (unsigned)__popc(acc));
-        if (nacc == 0)
-            break;
-        acc_any |= acc;
-        pend |= acc;
-        // a falling minimum lowers lim, so keep the largest lim of the pending cells
-        pl0 = lt(pl0, lim0) ? lim0 : pl0;
-        pl1 = lt(pl1, lim1) ? lim1 : pl1;
-        st.accepted += (unsigned long long)nacc;
-        if (++rounds > p.max_rounds) {
-            if (lane == 0)
-                atomicOr(&s.ctrl->error, ERR_ROUNDS);
-            break;
-        }
-        __syncwarp();
-        relax = neighbour_mask(acc, lane) & ~frozen & ~settled;
-    }
-
-    // ---- write back, front minima, overlap change notification ------------
-    // A boundary cell accepted here (and known at the end) is flagged to the
-    // neighbour only if the adjacent halo cell is not known with a value at or
-    // below it: such a neighbour cell can never take it as an upwind value
-    // (Algorithm 11 uses only smaller known neighbours, and values only
-    // decrease), so the exchange would change nothing there.
-    unsigned long long fo0 = 0, fo1 = 0, fo2 = 0, fo3 = 0, fo4 = 0, fo5 = 0;
-    real fv0 = INF, fv1 = INF;   // smallest flagged value per side
-    const unsigned chg = acc_any & known;
-    __syncwarp();   // the list buffer holds the tags again from here
-#pragma unroll 2
-    for (int k = 0; k < 16; ++k) {
-        const int c = lane + 32 * k;
-        const int ti = tb + 40 * (k & 1) + 100 * (k >> 1);
-        const real v = kval(W.kv[ti]);
-        uint8_t t;
-        if ((out >> k) & 1u)
-            t = TG_OUT | ST_FAR;
-        else if ((fix >> k) & 1u)
-            t = ST_FIX;
-        else if ((known >> k) & 1u)
-            t = ST_KNOWN;
-        else if ((band >> k) & 1u)
-            t = ST_BAND;
-        else
-            t = ST_FAR;
-        if ((neg >> k) & 1u)
-            t |= TG_NEG;
-        stag[c] = t;
-        if (kMode == 1 && ((chg >> k) & 1u)) {
-            const int y = lr + 4 * (k & 1), z = k >> 1;
-            bool flagged = false;
-            if (lx == 0 && lt(v, W.kv[ti - 1])) {
-                fo0 |= 1ull << (y + 8 * z);
-                flagged = true;
-            }
-            if (lx == 7 && lt(v, W.kv[ti + 1])) {
-                fo1 |= 1ull << (y + 8 * z);
-                flagged = true;
-            }
-            if (y == 0 && lt(v, W.kv[ti - kTile])) {
-                fo2 |= 1ull << (lx + 8 * z);
-                flagged = true;
-            }
-            if (y == 7 && lt(v, W.kv[ti + kTile])) {
-                fo3 |= 1ull << (lx + 8 * z);
-                flagged = true;
-            }
-            if (z == 0 && lt(v, W.kv[ti - kTile * kTile])) {
-                fo4 |= 1ull << (lx + 8 * y);
-                flagged = true;
-            }
-            if (z == 7 && lt(v, W.kv[ti + kTile * kTile])) {
-                fo5 |= 1ull << (lx + 8 * y);
-                flagged = true;
-            }
-            if (flagged) {
-                if ((neg >> k) & 1u)
-                    fv0 = vmin(fv0, v);
-                else
-                    fv1 = vmin(fv1, v);
-            }
-        }
-    }
-    // write back with 16-byte stores from the rows of the tile (marks cleared)
-    __syncwarp();
-    {
-        constexpr int kVecs = kB3 * (int)sizeof(real) / 16 / 32;
-        uint4 *gv = reinterpret_cast<uint4 *>(T + base);
-#pragma unroll
-        for (int j = 0; j < kVecs; ++j) {
-            const int q = lane + 32 * j;
-            gv[q] = row_load(W.kv, q);
-        }
-        reinterpret_cast<uint4 *>(tag + base)[lane] = reinterpret_cast<const uint4 *>(stag)[lane];
-        if (kTape)
-            reinterpret_cast<uint4 *>(s.tape + base)[lane] = reinterpret_cast<const uint4 *>(W.tp)[lane];
-    }
-    notify_v[0] = kMode == 1 ? warp_min(fv0) : INF;
-    notify_v[1] = kMode == 1 ? warp_min(fv1) : INF;
-    if (lane == 0) {
-        bmin[2 * b] = m0;
-        bmin[2 * b + 1] = m1;
-    }
-    notify_m = 0;
-    notify_nb = -1;
-    if (kMode == 1) {
-        unsigned long long m = 0;
-#define FMM_FACE_OR(f, val)                                                        \
-    {                                                                              \
-        const unsigned lo = __reduce_or_sync(FULL, (unsigned)(val));               \
-        const unsigned hi = __reduce_or_sync(FULL, (unsigned)((val) >> 32));       \
-        if (lane == (f))                                                           \
-            m = (unsigned long long)lo | ((unsigned long long)hi << 32);           \
-    }
-        FMM_FACE_OR(0, fo0) FMM_FACE_OR(1, fo1) FMM_FACE_OR(2, fo2)
-        FMM_FACE_OR(3, fo3) FMM_FACE_OR(4, fo4) FMM_FACE_OR(5, fo5)
-#undef FMM_FACE_OR
-#pragma unroll
-        for (int f = 0; f < kFaces; ++f)
-            if (lane == f)
-                notify_nb = nbi[f];
-        notify_m = (lane < kFaces && notify_nb >= 0) ? m : 0ull;
-        st.marches += 1;
-        st.rounds += (unsigned long long)rounds;
-    }
-}
 
 __device__ __forceinline__ void flush_stats(Control *ctrl, MarchStats &st, int lane)
 {
@@ -1141,41 +366,182 @@ __device__ __forceinline__ void flush_stats(Control *ctrl, MarchStats &st, int l
         atomicAdd(&ctrl->exchanges, (unsigned long long)ex);
     }
 }
+__device__ __forceinline__ unsigned long long vloadu(const unsigned long long *p)
+{
+    return *(const volatile unsigned long long *)p;
+}
+
+// Put brick b into ring slot t (waits, bounded, for a slot still being read).
+__device__ __forceinline__ void ring_put(Control *c, unsigned long long *q, unsigned long long cap,
+                                         unsigned long long t, long long b)
+{
+    const unsigned long long v = ((t & 0xffffffffull) << 32) | (unsigned long long)(b + 1);
+    unsigned long long *slot = q + (t % cap);
+    if (atomicCAS(slot, 0ull, v) == 0ull)
+        return;
+    const unsigned long long ts = device_ns(), lim = vload(&c->wait_ns);
+    while (atomicCAS(slot, 0ull, v) != 0ull) {
+        if (device_ns() - ts > lim || (vload((const int *)&c->error) & ERR_SPIN)) {
+            atomicOr(&c->error, ERR_SPIN);
+            break;
+        }
+        __nanosleep(32);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// The brick scheduler of the one-launch schedules.
+//
+// work[b] is one 64-bit word per brick: the smallest work the brick has (the
+// smallest changed halo value flagged to it, or its own smallest BAND value;
+// a float, rounded down) and two flags.  kWorkActive: the brick is in the
+// ready queue or being marched.  kWorkWaiting: the waiting ring holds an entry
+// of it.  Every transition is one atomic on that word, so a brick is queued
+// once, marched by one warp, and no change is lost:
+//   a march that changed a face lowers the neighbour's value and, if the
+//   neighbour is not active, makes it active and queues it (value at or below
+//   the bound) or leaves it in the waiting ring;
+//   the warp that pops a brick takes the value (+inf in its place) before it
+//   reads the halo, and at the end of the march a value that arrived
+//   meanwhile keeps the brick active or sends it to the ring.
+// ---------------------------------------------------------------------------
+constexpr unsigned kWorkActive = 1u, kWorkWaiting = 2u, kWorkFull = 4u, kWorkFace = 8u;
+constexpr unsigned kNoWork = 0x7f800000u;   // +inf
+
+__device__ __forceinline__ unsigned long long work_word(unsigned key, unsigned flags)
+{
+    return ((unsigned long long)key << 32) | flags;
+}
+__device__ __forceinline__ unsigned work_key(float v) { return __float_as_uint(v); }
+__device__ __forceinline__ unsigned work_key(double v) { return __float_as_uint(__double2float_rd(v)); }
+
+// Take brick b from the queue: forget the work recorded so far, then read its
+// halo (acquire: the cells behind the recorded values are visible).  Returns
+// the changed faces (bit f), all ones for kWorkFull.
+__device__ __forceinline__ unsigned take_brick(const DeviceState &s, long long b, int lane)
+{
+    unsigned fl = 0;
+    if (lane == 0) {
+        unsigned long long old = vloadu(&s.work[b]);
+        for (;;) {
+            const unsigned long long nw = work_word(kNoWork, (unsigned)old & (kWorkActive | kWorkWaiting));
+            unsigned long long was;
+            asm volatile("atom.acquire.gpu.global.cas.b64 %0, [%1], %2, %3;"
+                         : "=l"(was)
+                         : "l"(s.work + b), "l"(old), "l"(nw)
+                         : "memory");
+            if (was == old)
+                break;
+            old = was;
+        }
+        fl = (unsigned)old;
+    }
+    fl = __shfl_sync(FULL, fl, 0);
+    return (fl & kWorkFull) ? ~0u : fl / kWorkFace;
+}
+
+// The end of a march of brick b (written back by all lanes): lane f < 6 with a
+// changed face flags the neighbour, lane kFaces ends the brick's own march,
+// and the warp queues and rings what they claimed.  `bound` is the level the
+// marches start at (a stale one only delays a start), kAll: no level, every
+// flagged brick is queued.  `pending` changes once: the bricks queued less
+// this one, after ring entries are counted and before queue slots are filled,
+// so it reaches zero only with nothing queued, marching or unrecorded.
+template <typename real, bool kAll>
+__device__ __forceinline__ void finish_brick(const DeviceState &s, unsigned long long cap, double width, long long b,
+                                             const Notify<real> &nt, int lane)
+{
+    Control *c = s.ctrl;
+    float bound = __uint_as_float(kNoWork);
+    if (!kAll)
+        bound = *(const volatile float *)&c->level[(vloadu(&c->scan_word) >> 32) & 1u].bound;
+    fence_acq_rel();   // the write-back before the flags
+    __syncwarp();
+    long long tb = -1;        // the brick whose word this lane updates
+    unsigned key = kNoWork;   // work to record
+    if (nt.m) {
+        tb = nt.nb;
+        key = work_key(vmin(nt.v[0], nt.v[1]));
+    } else if (lane == kFaces) {
+        tb = b;
+        const real band = vmin(nt.band[0], nt.band[1]);
+        if (!kAll && (double)band <= width)
+            key = work_key(band);
+    }
+    int act = 0;   // 1: queue tb, 2: append it to the waiting ring
+    if (tb >= 0) {
+        unsigned long long old = vloadu(&s.work[tb]);
+        for (;;) {
+            const unsigned k = umin((unsigned)(old >> 32), key);
+            unsigned fl = (unsigned)old;
+            act = 0;
+            if (nt.m)
+                fl |= kWorkFace << (lane ^ 1);
+            else {
+                fl &= ~kWorkActive;
+                if (key < kNoWork)
+                    fl |= kWorkFull;
+            }
+            if (!(fl & kWorkActive) && k < kNoWork) {
+                if (__uint_as_float(k) <= bound) {
+                    fl |= kWorkActive;
+                    act = 1;
+                } else if (!(fl & kWorkWaiting)) {
+                    fl |= kWorkWaiting;
+                    act = 2;
+                }
+            }
+            const unsigned long long was = atomicCAS(&s.work[tb], old, work_word(k, fl));
+            if (was == old)
+                break;
+            old = was;
+        }
+    }
+    const unsigned bq = __ballot_sync(FULL, act == 1), bw = __ballot_sync(FULL, act == 2);
+    unsigned long long tq = 0, tw = 0;
+    if (lane == 0) {
+        const int n = __popc(bq);
+        if (bw)
+            tw = atomicAdd(&c->w_tail, (unsigned long long)__popc(bw));
+        if (n != 1) {
+            __threadfence();   // ring entries counted, words released
+            atomicAdd(&c->pending, n - 1);
+        }
+        if (n)
+            tq = atomicAdd(&c->q_tail, (unsigned long long)n);
+    }
+    if (bq | bw) {
+        tq = __shfl_sync(FULL, tq, 0);
+        tw = __shfl_sync(FULL, tw, 0);
+        const unsigned below = (1u << lane) - 1u;
+        if (act == 1)
+            ring_put(c, s.queue, cap, tq + __popc(bq & below), tb);
+        else if (act == 2)
+            ring_put(c, s.waiting, cap, tw + __popc(bw & below), tb);
+    }
+    __syncwarp();
+}
 
 // Phased march: kMode 0 runs Algorithm 9 over all bricks; kMode 1 runs
-// Algorithm 12 over the bricks of work list `which` (taken one at a time from
-// a shared counter) with the change masks the select kernel moved to the
-// inbox; changes are flagged in the neighbours' live masks and dirty flags.
+// Algorithm 12 up to the restart bound over the bricks of work list `which`
+// (taken one at a time from a shared counter); changes are flagged in the
+// neighbours' live masks and dirty flags.
 template <typename real, bool kHetero, int kMode, bool kTape, bool kAniso>
 __global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape>())
     k_march(Geom g, DeviceState s, SolveParams p, double spd_const_term, int which)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpTile<real, kTape> &W = reinterpret_cast<WarpTile<real, kTape> *>(smem_raw)[warp];
+    MarchSmem<real, kTape> &sm = *reinterpret_cast<MarchSmem<real, kTape> *>(smem_raw);
+    WarpTile<real, kTape> &W = sm.tile[warp];
     Control *ctrl = s.ctrl;
-    if (kMode == 1 && ctrl->done)
-        return;
-    const long long n = (kMode == 0) ? g.nbricks : (long long)ctrl->n_list[which];
-    // select the list without indexing the parameter struct at run time
-    // (that would copy the struct to local memory)
-    const int *work_list = which ? s.list[1] : s.list[0];
-    const real bound0 = (real)ctrl->bound[0], bound1 = (real)ctrl->bound[1];
-    MarchStats st = {0, 0, 0, 0, 0};
-    long long it = 0, next = 0;
-    if (kMode == 1) {
-        if (lane == 0) {
-            it = (long long)atomicAdd(&ctrl->work[which], 1u);
-            next = (long long)atomicAdd(&ctrl->work[which], 1u);
-        }
-        it = __shfl_sync(FULL, it, 0);
-        next = __shfl_sync(FULL, next, 0);
-    } else {
-        it = (long long)blockIdx.x * kMarchWarps + warp;
-    }
-    while (it < n) {
-        const long long b = (kMode == 0) ? it : (long long)work_list[it];
-        if (kMode == 0) {
+    if constexpr (kMode == 0) {
+        for (long long b = (long long)blockIdx.x * kMarchWarps + warp; b < g.nbricks;
+             b += (long long)gridDim.x * kMarchWarps) {
+            long long nbi[kFaces];
+#pragma unroll
+            for (int f = 0; f < kFaces; ++f)
+                nbi[f] = neighbour_brick(g, s.nbr, b, f);
             // Algorithm 9 only changes cells next to a FIX cell: a brick with
             // no FIX cell in it or in its six neighbours keeps the state of
             // Algorithm 8 and has no BAND cell (one 16-byte load of tags per
@@ -1183,7 +549,7 @@ __global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape
             bool fixnear = false;
 #pragma unroll
             for (int f = -1; f < kFaces; ++f) {
-                const long long q = f < 0 ? b : neighbour_brick(g, s.nbr, b, f);
+                const long long q = f < 0 ? b : nbi[f < 0 ? 0 : f];
                 if (q < 0)
                     continue;
                 const uint4 t4 = reinterpret_cast<const uint4 *>(s.tag + q * kB3)[lane];
@@ -1194,357 +560,157 @@ __global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape
             if (!__any_sync(FULL, fixnear)) {
                 if (lane < 2)
                     ((real *)s.bmin)[2 * b + lane] = inf_v<real>();
-                it += (long long)gridDim.x * kMarchWarps;
                 continue;
             }
+            front_brick<real, kHetero, kTape, kAniso>(s, p, spd_const_term, W, b, nbi, lane);
+            __syncwarp();
         }
-        unsigned long long F[kFaces];
+    } else {
+        if (ctrl->done)
+            return;
+        load_sweep_order(sm.order);
+        const long long n = (long long)ctrl->n_list[which];
+        // select the list without indexing the parameter struct at run time
+        // (that would copy the struct to local memory)
+        const int *work_list = which ? s.list[1] : s.list[0];
+        const real bound0 = (real)ctrl->bound[0], bound1 = (real)ctrl->bound[1];
+        MarchStats st = {0, 0, 0, 0, 0};
+        long long it = 0, next = 0;
+        if (lane == 0) {
+            it = (long long)atomicAdd(&ctrl->work[which], 1u);
+            next = (long long)atomicAdd(&ctrl->work[which], 1u);
+        }
+        it = __shfl_sync(FULL, it, 0);
+        next = __shfl_sync(FULL, next, 0);
+        while (it < n) {
+            const long long b = (long long)work_list[it];
+            long long nbi[kFaces];
 #pragma unroll
-        for (int f = 0; f < kFaces; ++f)
-            F[f] = kMode == 1 ? s.inbox[b * kFaces + f] : 0ull;
-        unsigned long long m;
-        long long nb;
-        real nv[2];
-        march_brick<real, kHetero, kMode, false, kTape, kAniso>(g, s, p, spd_const_term, W, b, F, bound0, bound1,
-                                                 lane, m, nb, nv, st);
-        if (kMode == 1 && m) {
-            atomicOr(&s.fresh[nb * kFaces + (lane ^ 1)], m);
-            s.dirty[nb] = 1u;
-            st.exchanges += (unsigned long long)__popcll(m);
-        }
-        __syncwarp();
-        if (kMode == 1) {
+            for (int f = 0; f < kFaces; ++f)
+                nbi[f] = neighbour_brick(g, s.nbr, b, f);
+            Notify<real> nt;
+            sweep_brick<real, kHetero, kTape, kAniso, true>(g, s, p, spd_const_term, sm.order, W, b, nbi, ~0u, bound0, bound1,
+                                                            lane, nt, st);
+            if (nt.m) {
+                s.dirty[nt.nb] = 1u;
+                st.exchanges += (unsigned long long)__popcll(nt.m);
+            }
+            __syncwarp();
             it = next;
             if (it < n && lane == 0)
                 next = (long long)atomicAdd(&ctrl->work[which], 1u);
             next = __shfl_sync(FULL, next, 0);
-        } else {
-            it += (long long)gridDim.x * kMarchWarps;
         }
-    }
-    if (kMode == 1)
         flush_stats(ctrl, st, lane);
-}
-
-// ---------------------------------------------------------------------------
-// Persistent restart: one launch marches every brick of a restart to the
-// bound until no brick has unconsumed halo changes.  Bricks wait in a ring
-// queue; a brick is in the queue or being marched at most once at a time
-// (queued[b] = 1 from the push until its march ends), so a brick always has a
-// single writer.  A march that changes boundary cells ORs them into the
-// neighbour's change masks after a fence and pushes the neighbour if it can
-// claim queued[nb]; a brick that ends its march clears queued[b] and pushes
-// itself again if masks arrived meanwhile.  `pending` counts bricks pushed and
-// not yet done; the launch ends when it reaches zero.  Every wait is bounded:
-// past the limit the kernel sets ERR_SPIN and returns.
-// ---------------------------------------------------------------------------
-
-template <typename real, bool kHetero, bool kTape, bool kAniso>
-__global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape>())
-    k_march_persistent(Geom g, DeviceState s, SolveParams p, double spd_const_term)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpTile<real, kTape> &W = reinterpret_cast<WarpTile<real, kTape> *>(smem_raw)[warp];
-    Control *ctrl = s.ctrl;
-    if (ctrl->done)
-        return;
-    const real bound0 = (real)ctrl->bound[0], bound1 = (real)ctrl->bound[1];
-    const unsigned long long cap = (unsigned long long)g.nbricks;
-    unsigned long long *q = s.queue;
-    MarchStats st = {0, 0, 0, 0, 0};
-    for (;;) {
-        long long b = -1;
-        if (lane == 0)
-            b = queue_pop(ctrl, q, cap);
-        b = __shfl_sync(FULL, b, 0);
-        if (b < 0)
-            break;
-        // take the changes flagged so far (later ones re-queue the brick)
-        unsigned long long mine = 0;
-        if (lane < kFaces)
-            mine = atomicExch(&s.fresh[b * kFaces + lane], 0ull);
-        __threadfence();
-        unsigned long long F[kFaces];
-#pragma unroll
-        for (int f = 0; f < kFaces; ++f)
-            F[f] = __shfl_sync(FULL, mine, f);
-        unsigned long long m;
-        long long nb;
-        real nv[2];
-        march_brick<real, kHetero, 1, true, kTape, kAniso>(g, s, p, spd_const_term, W, b, F, bound0, bound1,
-                                            lane, m, nb, nv, st);
-        // publish the write-back before flagging anything
-        __threadfence();
-        __syncwarp();
-        if (m) {
-            atomicOr(&s.fresh[nb * kFaces + (lane ^ 1)], m);
-            st.exchanges += (unsigned long long)__popcll(m);
-            // the mask must be visible before the claim: a brick that ends
-            // its march clears its flag and then re-reads its masks
-            __threadfence();
-            if (atomicCAS(&s.queued[nb], 0u, 1u) == 0u) {
-                atomicAdd(&ctrl->pending, 1);
-                queue_push(ctrl, q, cap, nb);
-            }
-        }
-        __syncwarp();
-        if (lane == 0) {
-            // end of the march: let neighbours queue the brick again, and do
-            // it here if changes arrived while it ran
-            atomicExch(&s.queued[b], 0u);
-            __threadfence();
-            bool again = false;
-#pragma unroll
-            for (int f = 0; f < kFaces; ++f)
-                again = again || (vload(&s.fresh[b * kFaces + f]) != 0ull);
-            if (again && atomicCAS(&s.queued[b], 0u, 1u) == 0u) {
-                atomicAdd(&ctrl->pending, 1);
-                queue_push(ctrl, q, cap, b);
-            }
-            __threadfence();
-            atomicAdd(&ctrl->pending, -1);
-        }
-        __syncwarp();
     }
-    flush_stats(ctrl, st, lane);
 }
 
 // ---------------------------------------------------------------------------
+// One-launch marches.  Warps take bricks from the ready queue until none is
+// queued or being marched.
+//
+// Persistent schedule (kAll): the bound of the restart is fixed, every flagged
+// brick is queued, the launch is one restart.
+//
 // Continuous schedule: the restarts of Algorithm 16 without the barrier
-// between them.  One launch marches until the solve is complete.  Each march
-// takes the current bound when it starts.  Once fewer bricks than raise_at
-// are queued or marching, an idle warp raises the bound to
-// max(bound, minimum seen by the last scan) + stride (at most width) and the
-// idle warps scan the per-brick minima in chunks, pushing every brick with a
-// BAND cell at or below the new bound; a brick that ends a march with a BAND
-// cell at or below the current bound pushes itself again.  The bricks of the
-// last shell of one restart thus overlap the first bricks of the next.  epoch
-// works as a sequence lock: odd while a raise rewrites the bound and the scan
-// counters.  The solve is complete when no raise is in progress, the last
-// scan is done, nothing is queued or marching and the bound has reached width
-// on both sides.  At the restart limit the raises stop and the launch ends
-// once the current level is drained, so the solve can be resumed from there.
-// Every wait is bounded (wait_ns without any progress).
+// between them, one launch for the whole solve.  The bound says which bricks
+// may start; a brick marches with the bound it finds (plus the look-ahead, by
+// default to its end).  Bricks whose work lies above the bound wait in a ring.
+// Once fewer bricks than raise_at are queued or marching, a warp raises the
+// bound to max(bound, smallest waiting value) + stride and the idle warps scan
+// the ring in chunks: bricks at or below the new bound are queued, the others
+// appended again.  Only bricks next to the front wait, so a raise touches a few
+// per cent of the bricks (scanning the minima of all bricks took 11% of the
+// 1024^3 march's warp time, and twice that waiting for the scans).  The solve
+// is complete when nothing is queued, marching, waiting or being scanned.  At
+// the restart limit the raises stop and the launch ends once the current
+// level is drained; the work words then say what is left.
+//
+// Every wait is bounded (wait_ns without any progress): past the limit the
+// kernel sets ERR_SPIN and returns.
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ double vloadd(const double *p) { return *(const volatile double *)p; }
-__device__ __forceinline__ unsigned long long vloadu(const unsigned long long *p)
+// Raise the bound (one lane).  Returns true when this warp raised it.
+__device__ bool try_raise(Control *c, const SolveParams &p, int pend)
 {
-    return *(const volatile unsigned long long *)p;
-}
-
-// Push, with one tail increment for the warp, the bricks b of the lanes whose
-// sel is set and that claim queued[b].
-__device__ __forceinline__ void queue_push_warp(Control *c, unsigned long long *q, unsigned long long cap,
-                                                unsigned *queued, long long b, bool sel, int lane)
-{
-    const bool mine = sel && atomicCAS(&queued[b], 0u, 1u) == 0u;
-    const unsigned ball = __ballot_sync(FULL, mine);
-    if (ball == 0u)
-        return;
-    unsigned long long t0 = 0;
-    if (lane == 0) {
-        atomicAdd(&c->pending, __popc(ball));
-        t0 = atomicAdd(&c->q_tail, (unsigned long long)__popc(ball));
-    }
-    t0 = __shfl_sync(FULL, t0, 0);
-    if (mine) {
-        const unsigned long long t = t0 + __popc(ball & ((1u << lane) - 1u));
-        const unsigned long long v = ((t & 0xffffffffull) << 32) | (unsigned long long)(b + 1);
-        unsigned long long *slot = q + (t % cap);
-        const unsigned long long ts = device_ns(), lim = vload(&c->wait_ns);
-        while (atomicCAS(slot, 0ull, v) != 0ull) {
-            if (device_ns() - ts > lim || (vload((const int *)&c->error) & ERR_SPIN)) {
-                atomicOr(&c->error, ERR_SPIN);
-                break;
-            }
-            __nanosleep(32);
-        }
-    }
-}
-
-// The smallest value neighbours flagged to brick side j (2 b + side) since it
-// last took its masks, +inf when none is recorded.
-constexpr unsigned long long kInminNone = ~0ull;
-template <typename real>
-__device__ __forceinline__ real inmin_bits(unsigned long long v)
-{
-    return v >= 0x7ff0000000000000ull ? inf_v<real>() : (real)__longlong_as_double((long long)v);
-}
-// both BAND minima of a brick (adjacent, 16- or 8-byte aligned) in one load
-__device__ __forceinline__ void ld_pair(const double *p, double &a, double &b)
-{
-    const double2 v = __ldcg(reinterpret_cast<const double2 *>(p));
-    a = v.x;
-    b = v.y;
-}
-__device__ __forceinline__ void ld_pair(const float *p, float &a, float &b)
-{
-    const float2 v = __ldcg(reinterpret_cast<const float2 *>(p));
-    a = v.x;
-    b = v.y;
-}
-
-template <typename real>
-__device__ __forceinline__ real inmin_value(const unsigned long long *inmin, long long j)
-{
-    const unsigned long long v = vloadu(inmin + j);
-    return v >= 0x7ff0000000000000ull ? inf_v<real>() : (real)__longlong_as_double((long long)v);
-}
-
-// One warp scans chunk ch of the per-brick minima for the bound (bd0, bd1).
-template <typename real>
-__device__ __forceinline__ void scan_chunk(const Geom &g, const DeviceState &s, int ch, real bd0,
-                                           real bd1, int lane)
-{
-    Control *c = s.ctrl;
-    const real *bmin = (const real *)s.bmin;
-    const real INF = inf_v<real>();
-    const unsigned long long cap = (unsigned long long)g.nbricks;
-    real l0 = INF, l1 = INF;
-    const long long first = (long long)ch * kScanChunk;
-    // kScanBatch bricks per lane at a time: both minima of a brick in one
-    // load, both flagged values in another, all loads of a batch in flight
-    // together (the scan is a chain of L2 round trips otherwise)
-    constexpr int kScanBatch = 2;
-    static_assert((kScanChunk / 32) % kScanBatch == 0, "whole batches per chunk");
-    for (int j0 = 0; j0 < kScanChunk / 32; j0 += kScanBatch) {
-        real bm[kScanBatch][2];
-        ulonglong2 im[kScanBatch];
-#pragma unroll
-        for (int u = 0; u < kScanBatch; ++u) {
-            const long long b = first + 32 * (j0 + u) + lane;
-            if (b < g.nbricks) {
-                ld_pair(bmin + 2 * b, bm[u][0], bm[u][1]);
-                im[u] = __ldcg(reinterpret_cast<const ulonglong2 *>(s.inmin + 2 * b));
-            } else {
-                bm[u][0] = bm[u][1] = INF;
-                im[u] = make_ulonglong2(kInminNone, kInminNone);
-            }
-        }
-#pragma unroll
-        for (int u = 0; u < kScanBatch; ++u) {
-            const long long b = first + 32 * (j0 + u) + lane;
-            const real m0 = vmin(bm[u][0], inmin_bits<real>(im[u].x));
-            const real m1 = vmin(bm[u][1], inmin_bits<real>(im[u].y));
-            l0 = vmin(l0, m0);
-            l1 = vmin(l1, m1);
-            const bool sel = b < g.nbricks && ((lt(m0, INF) && !lt(bd0, m0)) || (lt(m1, INF) && !lt(bd1, m1)));
-            queue_push_warp(c, s.queue, cap, s.queued, b, sel, lane);
-        }
-    }
-    l0 = warp_min(l0);
-    l1 = warp_min(l1);
-    if (lane == 0) {
-        atomicMin(&c->scan_min[0], (unsigned long long)__double_as_longlong((double)l0));
-        atomicMin(&c->scan_min[1], (unsigned long long)__double_as_longlong((double)l1));
-        __threadfence();
-        atomicAdd(&c->scan_done, 1);
-    }
-}
-
-// Raise the bound (lane 0).  Returns true when this warp raised it.  For each
-// side, with m the smallest BAND minimum the last scan saw, the new bound is
-// max(bound, m) + stride, but while bricks are queued or marching at most
-// max_lead strides above floor(m / stride) * stride, so a small front
-// cannot run ahead.  A scan that saw no BAND cell on a side proves the side
-// finished only if it started with nothing queued or marching (a clean
-// scan): otherwise the side's next BAND cells may have been in flight, in
-// bricks notified but not yet marched, and the side waits while bricks are
-// in flight, or rises by one stride (which starts a clean scan) when none
-// are.  With nothing queued or marching every BAND value is above the
-// bound, so the bound always rises.
-__device__ bool try_raise(Control *c, const SolveParams &p, int nchunks, int pend)
-{
-    const int e = vload(&c->epoch);
-    if ((e & 1) || vload(&c->scan_done) < nchunks)
+    const unsigned long long w = vloadu(&c->scan_word);
+    const int ep = (int)(w >> 32);
+    const auto *lv = &c->level[ep & 1];
+    if (vload(&c->scan_done) < vload(&lv->nchunks) || vloadu(&c->w_tail) == vloadu(&c->w_head))
         return false;
-    const double b0 = vloadd(&c->bound[0]), b1 = vloadd(&c->bound[1]);
-    if (b0 >= p.width && b1 >= p.width)
+    if (atomicCAS(&c->raise_lock, ep, ep + 1) != ep)
         return false;
-    double nb[2];
-    const double bo[2] = {b0, b1};
-#pragma unroll
-    for (int sd = 0; sd < 2; ++sd) {
-        const double sm = __longlong_as_double((long long)vloadu(&c->scan_min[sd]));
-        double v;
-        if (!(sm < CUDART_INF)) {
-            if (pend > 0)
-                v = bo[sd];
-            else if (vload(&c->scan_clean))
-                v = p.width;
-            else
-                v = fmin(bo[sd] + p.stride, p.width);
-        } else {
-            v = fmax(bo[sd], sm) + p.stride;
-            if (pend > 0 && p.stride < CUDART_INF)
-                v = fmin(v, (floor(sm / p.stride) + p.max_lead) * p.stride);
-            v = fmin(v, p.width);
-        }
-        nb[sd] = fmax(v, bo[sd]);
-    }
-    if (!(nb[0] > b0 || nb[1] > b1))
-        return false;
-    if (atomicCAS(&c->epoch, e, e + 1) != e)
-        return false;
-    if (p.max_restarts > 0 && (long long)vload(&c->restart) >= p.max_restarts) {
+    __threadfence();
+    const unsigned long long base = vloadu(&c->w_head), end = vloadu(&c->w_tail);
+    bool ok = end != base && vload(&c->scan_done) >= vload(&lv->nchunks);
+    if (ok && p.max_restarts > 0 && (long long)vload(&c->restart) >= p.max_restarts) {
         // the restart limit counts the raises too
         atomicOr(&c->error, ERR_RESTARTS);
+        ok = false;
+    }
+    if (!ok) {
         __threadfence();
-        atomicExch(&c->epoch, e + 2);
+        atomicExch(&c->raise_lock, ep);
         return false;
     }
-    atomicExch(&c->scan_done, 0);
-    atomicExch(&c->scan_clean, pend == 0 ? 1 : 0);
+    const float b0 = *(const volatile float *)&lv->bound;
+    const float sm = __uint_as_float(*(const volatile unsigned *)&c->scan_min);
+    double v = (double)(sm < CUDART_INF_F ? fmaxf(b0, sm) : b0) + p.stride;
+    if (pend > 0 && p.stride < CUDART_INF && sm < CUDART_INF_F)
+        v = fmin(v, (floor((double)sm / p.stride) + p.max_lead) * p.stride);
+    const float nb = fmaxf(__double2float_ru(fmin(v, p.width)), b0);
+    const unsigned count = (unsigned)(end - base);
+    const int warps = gridDim.x * kMarchWarps;
+    int chunk = (int)((count + warps - 1) / warps);
+    chunk = (chunk + 31) & ~31;
+    auto *nl = &c->level[(ep + 1) & 1];
+    *(volatile unsigned long long *)&nl->base = base;
+    *(volatile unsigned long long *)&nl->end = end;
+    *(volatile int *)&nl->chunk = chunk;
+    *(volatile int *)&nl->nchunks = (int)((count + chunk - 1) / chunk);
+    *(volatile float *)&nl->bound = nb;
+    *(volatile unsigned long long *)&c->w_head = end;
+    *(volatile int *)&c->scan_done = 0;
+    *(volatile unsigned *)&c->scan_min = kNoWork;
+    *(volatile int *)&c->restart = vload(&c->restart) + 1;
     __threadfence();
-    *(volatile double *)&c->bound[0] = nb[0];
-    *(volatile double *)&c->bound[1] = nb[1];
-    atomicExch(&c->scan_min[0], 0x7ff0000000000000ull);
-    atomicExch(&c->scan_min[1], 0x7ff0000000000000ull);
-    atomicAdd(&c->restart, 1);
-    __threadfence();
-    atomicExch(&c->scan_next, 0);
-    __threadfence();
-    atomicExch(&c->epoch, e + 2);
+    atomicExch(&c->scan_word, (unsigned long long)(ep + 1) << 32);
     return true;
 }
 
-// The solve is complete (lane 0; see above).
-// The launch ends when the solve is complete or, once the restart limit has
-// stopped the raises (limited), when the current level is drained: no raise
-// or scan in progress and nothing queued or marching.  The state is then the
-// one after a restart of Algorithm 16, from which a solve can resume.
-__device__ bool launch_done(Control *c, const SolveParams &p, int nchunks, bool limited)
+// Nothing is queued, marching, waiting or being scanned (one lane; limited:
+// nothing but waiting).
+__device__ bool launch_done(Control *c, bool limited)
 {
-    const int e = vload(&c->epoch);
-    if ((e & 1) || vload(&c->scan_done) < nchunks)
+    const int ep = (int)(vloadu(&c->scan_word) >> 32);
+    if (vload(&c->scan_done) < vload(&c->level[ep & 1].nchunks))
         return false;
     __threadfence();
     if (vload(&c->pending) != 0)
         return false;
-    if (!limited && (vloadd(&c->bound[0]) < p.width || vloadd(&c->bound[1]) < p.width))
+    __threadfence();
+    if (!limited && vloadu(&c->w_tail) != vloadu(&c->w_head))
         return false;
     __threadfence();
-    return vload(&c->epoch) == e;
+    return vload(&c->raise_lock) == ep && (int)(vloadu(&c->scan_word) >> 32) == ep &&
+           vload(&c->scan_done) >= vload(&c->level[ep & 1].nchunks);
 }
 
-// Lane 0: the next job of the warp.  job 0: march brick arg; 1: scan chunk
-// arg; 2: stop.  ticket is the queue ticket the warp holds (-1: none).
-__device__ void next_job(Control *c, unsigned long long *q, unsigned long long cap,
-                         const SolveParams &p, int nchunks, long long &ticket, int &job,
-                         long long &arg)
+// One lane: the next job of the warp.  job 0: march brick arg; 1: scan chunk
+// arg of raise `ep`; 2: stop.  ticket is the queue ticket the warp holds (-1:
+// none).  A warp polls its own queue slot; the words every warp shares are read
+// by one warp of the CTA every time and by the others every eighth time.
+template <bool kAll>
+__device__ void next_job(Control *c, unsigned long long *q, unsigned long long cap, const SolveParams &p, bool leader,
+                         long long &ticket, int &job, long long &arg, int &ep_out)
 {
     if (ticket < 0)
         ticket = (long long)atomicAdd(&c->q_head, 1ull);
     unsigned long long *slot = q + ((unsigned long long)ticket % cap);
     const unsigned long long want = (unsigned long long)ticket & 0xffffffffull;
-    unsigned long long t0 = device_ns();
-    unsigned long long seen_tail = vloadu(&c->q_tail);
-    const unsigned long long lim = vloadu(&c->wait_ns);
-    int seen_done = vload(&c->scan_done), seen_epoch = vload(&c->epoch);
-    unsigned ns = 64;
-    for (;;) {
+    unsigned long long t0 = 0, seen = ~0ull;
+    unsigned ns = 32, tick = leader ? 0u : (unsigned)ticket & 7u;
+    for (;; ++tick) {
         const unsigned long long v = vloadu(slot);
         if (v != 0ull && (v >> 32) == want) {
             atomicExch(slot, 0ull);
@@ -1553,214 +719,252 @@ __device__ void next_job(Control *c, unsigned long long *q, unsigned long long c
             arg = (long long)(v & 0xffffffffull) - 1;
             return;
         }
-        const int err = vload(&c->error);
-        if (err & ERR_SPIN) {
-            job = 2;
-            return;
-        }
-        const bool limited = (err & ERR_RESTARTS) != 0;
-        if (vload(&c->scan_next) < nchunks) {
-            const int ch = atomicAdd(&c->scan_next, 1);
-            if (ch < nchunks) {
-                job = 1;
-                arg = ch;
+        if (leader || (tick & 7u) == 7u) {
+            const int err = vload(&c->error);
+            if (err & ERR_SPIN) {
+                job = 2;
                 return;
             }
-        }
-        const int pend = vload(&c->pending);
-        if (!limited && pend < p.raise_at && try_raise(c, p, nchunks, pend))
-            continue;
-        if (pend == 0 && launch_done(c, p, nchunks, limited)) {
-            job = 2;
-            return;
-        }
-        const unsigned long long now = device_ns(), tail = vloadu(&c->q_tail);
-        const int dn = vload(&c->scan_done), ep = vload(&c->epoch);
-        if (tail != seen_tail || dn != seen_done || ep != seen_epoch) {
-            seen_tail = tail;
-            seen_done = dn;
-            seen_epoch = ep;
-            t0 = now;
-        } else if (now - t0 > lim) {
-            break;
+            const bool limited = (err & ERR_RESTARTS) != 0;
+            const int pend = vload(&c->pending);
+            unsigned long long w = vloadu(&c->scan_word);
+            if (!kAll) {
+                if ((int)(unsigned)w < vload(&c->level[(w >> 32) & 1u].nchunks)) {
+                    w = atomicAdd(&c->scan_word, 1ull);
+                    __threadfence();   // the level this chunk belongs to
+                    ep_out = (int)(w >> 32);
+                    if ((int)(unsigned)w < vload(&c->level[ep_out & 1].nchunks)) {
+                        job = 1;
+                        arg = (long long)(unsigned)w;
+                        return;
+                    }
+                }
+                if (!limited && pend < p.raise_at && try_raise(c, p, pend))
+                    continue;
+            }
+            if (pend == 0 && launch_done(c, limited || kAll)) {
+                job = 2;
+                return;
+            }
+            // progress: a push, a raise or a scanned chunk
+            const unsigned long long mark = vloadu(&c->q_tail) + (w << 8) + (unsigned)vload(&c->scan_done);
+            const unsigned long long now = device_ns();
+            if (mark != seen) {
+                seen = mark;
+                t0 = now;
+            } else if (now - t0 > vloadu(&c->wait_ns)) {
+                break;
+            }
         }
         __nanosleep(ns);
-        if (ns < 2048)
+        if (ns < 256)
             ns <<= 1;
     }
     atomicOr(&c->error, ERR_SPIN);
     job = 2;
 }
 
-template <typename real, bool kHetero, bool kTape, bool kAniso>
-__global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape>())
-    k_march_continuous(Geom g, DeviceState s, SolveParams p, double spd_const_term)
+// One warp scans a chunk of the waiting ring for the bound of raise ep.
+__device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long long cap, int ch, int ep, int lane)
 {
+    Control *c = s.ctrl;
+    const auto &lv = c->level[ep & 1];
+    const unsigned long long end = vloadu(&lv.end);
+    const int chunk = vload(&lv.chunk);
+    const float bound = *(const volatile float *)&lv.bound;
+    const unsigned long long first = vloadu(&lv.base) + (unsigned long long)ch * (unsigned)chunk;
+    unsigned kept = kNoWork;
+    for (int i = 0; i < chunk; i += 32) {
+        const unsigned long long pos = first + (unsigned)(i + lane);
+        long long b = -1;
+        if (pos < end) {
+            // the entry may still be on its way from the warp that counted it
+            unsigned long long *slot = s.waiting + pos % cap;
+            const unsigned long long want = pos & 0xffffffffull;
+            unsigned long long v = vloadu(slot);
+            if (v == 0ull || (v >> 32) != want) {
+                const unsigned long long ts = device_ns(), lim = vloadu(&c->wait_ns);
+                while (v == 0ull || (v >> 32) != want) {
+                    if (device_ns() - ts > lim || (vload(&c->error) & ERR_SPIN)) {
+                        atomicOr(&c->error, ERR_SPIN);
+                        break;
+                    }
+                    __nanosleep(32);
+                    v = vloadu(slot);
+                }
+            }
+            if (v != 0ull && (v >> 32) == want) {
+                atomicExch(slot, 0ull);
+                b = (long long)(v & 0xffffffffull) - 1;
+            }
+        }
+        int act = 0;   // 1: queue, 2: keep waiting
+        if (b >= 0) {
+            unsigned long long old = vloadu(&s.work[b]);
+            for (;;) {
+                const unsigned k = (unsigned)(old >> 32);
+                unsigned fl = (unsigned)old;
+                act = 0;
+                if (!(fl & kWorkActive) && k < kNoWork) {
+                    if (__uint_as_float(k) > bound) {
+                        act = 2;
+                        kept = umin(kept, k);
+                        break;
+                    }
+                    fl |= kWorkActive;
+                    act = 1;
+                }
+                const unsigned long long was = atomicCAS(&s.work[b], old, work_word(k, fl & ~kWorkWaiting));
+                if (was == old)
+                    break;
+                old = was;
+            }
+        }
+        const unsigned bq = __ballot_sync(FULL, act == 1), bw = __ballot_sync(FULL, act == 2);
+        unsigned long long tq = 0, tw = 0;
+        if (lane == 0) {
+            if (bq) {
+                atomicAdd(&c->pending, __popc(bq));
+                tq = atomicAdd(&c->q_tail, (unsigned long long)__popc(bq));
+            }
+            if (bw)
+                tw = atomicAdd(&c->w_tail, (unsigned long long)__popc(bw));
+        }
+        tq = __shfl_sync(FULL, tq, 0);
+        tw = __shfl_sync(FULL, tw, 0);
+        const unsigned below = (1u << lane) - 1u;
+        if (act == 1)
+            ring_put(c, s.queue, cap, tq + __popc(bq & below), b);
+        else if (act == 2)
+            ring_put(c, s.waiting, cap, tw + __popc(bw & below), b);
+    }
+    kept = __reduce_min_sync(FULL, kept);
+    if (lane == 0) {
+        if (kept < kNoWork)
+            atomicMin(&c->scan_min, kept);
+        __threadfence();
+        atomicAdd(&c->scan_done, 1);
+    }
+    __syncwarp();
+}
+
+template <typename real, bool kHetero, bool kTape, bool kAniso, bool kBounded, bool kAll>
+__global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape>())
+    k_march_queue(Geom g, DeviceState s, SolveParams p, double spd_const_term)
+{
+    static_assert(kBounded || !kAll, "a restart with a fixed bound is a bounded march");
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    WarpTile<real, kTape> &W = reinterpret_cast<WarpTile<real, kTape> *>(smem_raw)[warp];
+    MarchSmem<real, kTape> &sm = *reinterpret_cast<MarchSmem<real, kTape> *>(smem_raw);
+    WarpTile<real, kTape> &W = sm.tile[warp];
     Control *ctrl = s.ctrl;
     if (ctrl->done)
         return;
+    load_sweep_order(sm.order);
     const unsigned long long cap = (unsigned long long)g.nbricks;
-    const int nchunks = (int)((g.nbricks + kScanChunk - 1) / kScanChunk);
-    const real *bmin = (const real *)s.bmin;
-    unsigned long long *q = s.queue;
+    const real INF = inf_v<real>();
     MarchStats st = {0, 0, 0, 0, 0};
     long long ticket = -1;
     for (;;) {
-        int job = 2;
+        int job = 2, ep = 0;
         long long arg = 0;
         if (lane == 0)
-            next_job(ctrl, q, cap, p, nchunks, ticket, job, arg);
+            next_job<kAll>(ctrl, s.queue, cap, p, warp == 0, ticket, job, arg, ep);
         job = __shfl_sync(FULL, job, 0);
         arg = __shfl_sync(FULL, arg, 0);
         if (job == 2)
             break;
         if (job == 1) {
-            real bd0 = 0, bd1 = 0;
-            if (lane == 0) {
-                bd0 = (real)vloadd(&ctrl->bound[0]);
-                bd1 = (real)vloadd(&ctrl->bound[1]);
-            }
-            bd0 = __shfl_sync(FULL, bd0, 0);
-            bd1 = __shfl_sync(FULL, bd1, 0);
-            scan_chunk<real>(g, s, (int)arg, bd0, bd1, lane);
+            ep = __shfl_sync(FULL, ep, 0);
+            scan_chunk(s, cap, (int)arg, ep, lane);
             continue;
         }
         const long long b = arg;
-        // forget the smallest flagged value, then take the masks: a value
-        // flagged in between is lost, and a brick with masks but no value
-        // counts as ready (below)
-        if (lane < 2)
-            atomicExch(&s.inmin[2 * b + lane], kInminNone);
-        __threadfence();
-        __syncwarp();
-        unsigned long long mine = 0;
-        if (lane < kFaces)
-            mine = atomicExch(&s.fresh[b * kFaces + lane], 0ull);
-        real bound0 = 0, bound1 = 0;
-        if (lane == 0) {
-            // accept up to the bound plus the look-ahead, never beyond
-            // width_band (cells above it stay BAND, Algorithm 12)
-            bound0 = (real)fmin(vloadd(&ctrl->bound[0]) + p.ahead, p.width);
-            bound1 = (real)fmin(vloadd(&ctrl->bound[1]) + p.ahead, p.width);
-        }
-        __threadfence();
-        bound0 = __shfl_sync(FULL, bound0, 0);
-        bound1 = __shfl_sync(FULL, bound1, 0);
-        unsigned long long F[kFaces];
+        long long nbi[kFaces];
 #pragma unroll
         for (int f = 0; f < kFaces; ++f)
-            F[f] = __shfl_sync(FULL, mine, f);
-        unsigned long long m;
-        long long nb;
-        real nv[2];
-        march_brick<real, kHetero, 1, true, kTape, kAniso>(g, s, p, spd_const_term, W, b, F, bound0, bound1,
-                                            lane, m, nb, nv, st);
-        __threadfence();
-        __syncwarp();
-        if (m) {
-            // the value first, then the mask: a brick that sees the mask
-            // also sees a value at most this one (or none, see above)
-            const real INF = inf_v<real>();
-            if (lt(nv[0], INF))
-                atomicMin(&s.inmin[2 * nb], (unsigned long long)__double_as_longlong((double)nv[0]));
-            if (lt(nv[1], INF))
-                atomicMin(&s.inmin[2 * nb + 1], (unsigned long long)__double_as_longlong((double)nv[1]));
-            __threadfence();
-            atomicOr(&s.fresh[nb * kFaces + (lane ^ 1)], m);
-            st.exchanges += (unsigned long long)__popcll(m);
-            __threadfence();
-            // the neighbour starts now if what it was sent is at or below
-            // the bound; otherwise the scan of a later bound pushes it
-            const real cb0 = (real)vloadd(&ctrl->bound[0]), cb1 = (real)vloadd(&ctrl->bound[1]);
-            const bool ready = (lt(nv[0], INF) && !lt(cb0, nv[0])) || (lt(nv[1], INF) && !lt(cb1, nv[1]));
-            if (ready && atomicCAS(&s.queued[nb], 0u, 1u) == 0u) {
-                atomicAdd(&ctrl->pending, 1);
-                queue_push(ctrl, q, cap, nb);
-            }
+            nbi[f] = neighbour_brick(g, s.nbr, b, f);
+        const unsigned dirty = take_brick(s, b, lane);
+        real bound0 = INF, bound1 = INF;
+        if (kAll) {
+            bound0 = (real)ctrl->bound[0];
+            bound1 = (real)ctrl->bound[1];
+        } else if (kBounded) {
+            // accept up to the bound plus the look-ahead, never beyond
+            // width_band (cells above it stay BAND, Algorithm 12)
+            const float bd = *(const volatile float *)&ctrl->level[(vloadu(&ctrl->scan_word) >> 32) & 1u].bound;
+            bound0 = bound1 = (real)fmin((double)__shfl_sync(FULL, bd, 0) + p.ahead, p.width);
         }
-        __syncwarp();
-        if (lane == 0) {
-            const real INF = inf_v<real>();
-            const real m0 = bmin[2 * b], m1 = bmin[2 * b + 1];
-            // end of the march: let others queue the brick again, and do it
-            // here if changes at or below the bound arrived meanwhile (or
-            // changes without a recorded value) or the bound has risen above
-            // one of its BAND minima
-            atomicExch(&s.queued[b], 0u);
-            __threadfence();
-            bool flagged = false;
-#pragma unroll
-            for (int f = 0; f < kFaces; ++f)
-                flagged = flagged || (vload(&s.fresh[b * kFaces + f]) != 0ull);
-            const real nb0 = (real)vloadd(&ctrl->bound[0]), nb1 = (real)vloadd(&ctrl->bound[1]);
-            bool again = false;
-            if (flagged) {
-                const unsigned long long i0 = vloadu(&s.inmin[2 * b]), i1 = vloadu(&s.inmin[2 * b + 1]);
-                const real v0 = inmin_value<real>(s.inmin, 2 * b), v1 = inmin_value<real>(s.inmin, 2 * b + 1);
-                again = (i0 == kInminNone && i1 == kInminNone) || (lt(v0, INF) && !lt(nb0, v0)) ||
-                        (lt(v1, INF) && !lt(nb1, v1));
-            }
-            again = again || (lt(m0, INF) && !lt(nb0, m0)) || (lt(m1, INF) && !lt(nb1, m1));
-            if (again && atomicCAS(&s.queued[b], 0u, 1u) == 0u) {
-                atomicAdd(&ctrl->pending, 1);
-                queue_push(ctrl, q, cap, b);
-            }
-            __threadfence();
-            atomicAdd(&ctrl->pending, -1);
-        }
-        __syncwarp();
+        Notify<real> nt;
+        sweep_brick<real, kHetero, kTape, kAniso, kBounded>(g, s, p, spd_const_term, sm.order, W, b, nbi, dirty,
+                                                            bound0, bound1, lane, nt, st);
+        st.exchanges += (unsigned long long)__popcll(nt.m);
+        finish_brick<real, kAll>(s, cap, p.width, b, nt, lane);
     }
     flush_stats(ctrl, st, lane);
 }
 
-// Seed the queue of a restart: bricks with a BAND cell at or below the bound.
+// Seed a launch: the work word of every brick from its BAND minima and the
+// work a stopped launch left, queued (at or below the bound) or waiting.
+// all: the bound of each side is fixed and nothing waits.
 template <typename real>
-__global__ void k_seed(Geom g, const real *__restrict__ bmin, const unsigned long long *inmin,
-                       Control *ctrl, unsigned *queued, unsigned long long *q)
+__global__ void k_seed(Geom g, const real *__restrict__ bmin, Control *ctrl, unsigned long long *work,
+                       unsigned long long *q, unsigned long long *waiting, double width, bool all)
 {
     if (ctrl->done)
         return;
+    const double bd0 = ctrl->bound[0], bd1 = ctrl->bound[1];
+    const float bd = __double2float_ru(fmin(bd0, bd1));
     if (blockIdx.x == 0 && threadIdx.x == 0) {
-        // no scan in progress (the continuous schedule raises the bound later)
-        const int nchunks = (int)((g.nbricks + kScanChunk - 1) / kScanChunk);
-        ctrl->epoch = 0;
-        ctrl->scan_next = nchunks;
-        ctrl->scan_done = nchunks;
-        ctrl->scan_clean = 0;
+        // level 0: no scan, the bound of k_control
+        ctrl->level[0].base = ctrl->level[0].end = 0ull;
+        ctrl->level[0].nchunks = 0;
+        ctrl->level[0].chunk = 32;
+        ctrl->level[0].bound = bd;
+        ctrl->scan_min = __float_as_uint(bd);
         if (ctrl->hold)
             atomicAdd(&ctrl->pending, 1);   // testing: the queue never drains
-        // as if a scan had seen the bound itself: the first raise adds one stride
-        ctrl->scan_min[0] = (unsigned long long)__double_as_longlong(ctrl->bound[0]);
-        ctrl->scan_min[1] = (unsigned long long)__double_as_longlong(ctrl->bound[1]);
     }
-    const double bd0 = ctrl->bound[0], bd1 = ctrl->bound[1];
     const int lane = threadIdx.x & 31;
     for (long long b0 = blockIdx.x * (long long)blockDim.x; b0 < g.nbricks;
          b0 += (long long)gridDim.x * blockDim.x) {
         const long long b = b0 + threadIdx.x;
-        bool sel = false;
+        int act = 0;
         if (b < g.nbricks) {
-            const double m0 = fmin((double)bmin[2 * b], inmin_value<double>(inmin, 2 * b));
-            const double m1 = fmin((double)bmin[2 * b + 1], inmin_value<double>(inmin, 2 * b + 1));
-            sel = (m0 < CUDART_INF && m0 <= bd0) || (m1 < CUDART_INF && m1 <= bd1);
+            const unsigned k0 = (unsigned)(work[b] >> 32);
+            const real m0 = bmin[2 * b], m1 = bmin[2 * b + 1];
+            unsigned key = k0 < kNoWork ? k0 : kNoWork;
+            if (all) {
+                // a flagged value was accepted by the neighbour: it is at or
+                // below the bound of its side or of an earlier restart
+                if (key < kNoWork || (lt(m0, inf_v<real>()) && (double)m0 <= bd0) ||
+                    (lt(m1, inf_v<real>()) && (double)m1 <= bd1))
+                    act = 1;
+            } else {
+                const real m = vmin(m0, m1);
+                if (lt(m, inf_v<real>()) && (double)m <= width)
+                    key = umin(key, work_key(m));
+                if (key < kNoWork)
+                    act = __uint_as_float(key) <= bd ? 1 : 2;
+            }
+            work[b] = work_word(key, kWorkFull | (act == 1 ? kWorkActive : (act == 2 ? kWorkWaiting : 0u)));
         }
-        const unsigned ball = __ballot_sync(0xffffffffu, sel);
-        if (ball == 0u)
-            continue;
-        unsigned long long basepos = 0;
+        const unsigned bq = __ballot_sync(FULL, act == 1), bw = __ballot_sync(FULL, act == 2);
+        unsigned long long tq = 0, tw = 0;
         if (lane == 0) {
-            basepos = atomicAdd(&ctrl->q_tail, (unsigned long long)__popc(ball));
-            atomicAdd(&ctrl->pending, __popc(ball));
+            if (bq) {
+                atomicAdd(&ctrl->pending, __popc(bq));
+                tq = atomicAdd(&ctrl->q_tail, (unsigned long long)__popc(bq));
+            }
+            if (bw)
+                tw = atomicAdd(&ctrl->w_tail, (unsigned long long)__popc(bw));
         }
-        basepos = __shfl_sync(0xffffffffu, basepos, 0);
-        if (sel) {
-            const unsigned long long t = basepos + __popc(ball & ((1u << lane) - 1u));
-            queued[b] = 1u;
-            q[t % (unsigned long long)g.nbricks] = ((t & 0xffffffffull) << 32) | (unsigned long long)(b + 1);
-        }
+        tq = __shfl_sync(FULL, tq, 0) + __popc(bq & ((1u << lane) - 1u));
+        tw = __shfl_sync(FULL, tw, 0) + __popc(bw & ((1u << lane) - 1u));
+        if (act == 1)
+            q[tq] = ((tq & 0xffffffffull) << 32) | (unsigned long long)(b + 1);
+        else if (act == 2)
+            waiting[tw] = ((tw & 0xffffffffull) << 32) | (unsigned long long)(b + 1);
     }
 }
 
@@ -1769,7 +973,7 @@ __global__ void k_seed(Geom g, const real *__restrict__ bmin, const unsigned lon
 // ---------------------------------------------------------------------------
 
 template <typename real>
-__global__ void k_reduce(Geom g, const real *__restrict__ bmin, const unsigned long long *inmin,
+__global__ void k_reduce(Geom g, const real *__restrict__ bmin, const unsigned long long *__restrict__ work,
                          const unsigned *__restrict__ dirty, Control *ctrl)
 {
     if (ctrl->done)
@@ -1780,8 +984,11 @@ __global__ void k_reduce(Geom g, const real *__restrict__ bmin, const unsigned l
     unsigned cnt = 0;
     for (long long b = blockIdx.x * (long long)blockDim.x + threadIdx.x; b < g.nbricks;
          b += (long long)gridDim.x * blockDim.x) {
-        m0 = fmin(m0, fmin((double)bmin[2 * b], inmin_value<double>(inmin, 2 * b)));
-        m1 = fmin(m1, fmin((double)bmin[2 * b + 1], inmin_value<double>(inmin, 2 * b + 1)));
+        m0 = fmin(m0, (double)bmin[2 * b]);
+        // work a stopped launch left: its side is not recorded
+        const unsigned key = (unsigned)(work[b] >> 32);
+        m1 = fmin(m1, key < kNoWork ? fmin((double)__uint_as_float(key), (double)bmin[2 * b + 1])
+                                    : (double)bmin[2 * b + 1]);
         cnt += dirty[b] != 0u;
     }
     m0 = warp_min(m0);
@@ -1807,6 +1014,17 @@ __global__ void k_reduce(Geom g, const real *__restrict__ bmin, const unsigned l
         if (cnt)
             atomicAdd(&ctrl->dirty_count, cnt);
     }
+}
+
+// empty queue and waiting ring, no raise or scan under way
+__device__ __forceinline__ void reset_queue(Control *c)
+{
+    c->q_head = c->q_tail = 0ull;
+    c->w_head = c->w_tail = 0ull;
+    c->pending = 0;
+    c->scan_word = 0ull;
+    c->scan_done = 0;
+    c->raise_lock = 0;
 }
 
 __global__ void k_control(Control *c, double width, double stride, long long max_restarts)
@@ -1838,21 +1056,16 @@ __global__ void k_control(Control *c, double width, double stride, long long max
     c->n_list[1] = 0u;
     c->work[0] = 0u;
     c->work[1] = 0u;
-    c->q_head = 0ull;
-    c->q_tail = 0ull;
-    c->pending = 0;
+    reset_queue(c);
 }
 
 // Work lists: list 0 = bricks with a BAND cell at or below the bound or with
 // pending overlap changes (first march); list 1 = bricks with pending changes
-// (second march, after the exchange).  A selected brick's change masks are
-// moved to its inbox here, between kernels, so the march reads them without
-// atomics; changes flagged during the march accumulate in the live masks for
-// the next selection.
+// (second march, after the exchange).  Changes flagged during the march are
+// left for the next selection.
 template <typename real>
 __global__ void k_select(Geom g, const real *__restrict__ bmin, unsigned *dirty,
-                         unsigned long long *fresh, unsigned long long *inbox, Control *ctrl,
-                         int *list, int which)
+                         Control *ctrl, int *list, int which)
 {
     if (ctrl->done)
         return;
@@ -1873,16 +1086,8 @@ __global__ void k_select(Geom g, const real *__restrict__ bmin, unsigned *dirty,
                 sel = sel || (m0 < CUDART_INF && m0 <= bd0) || (m1 < CUDART_INF && m1 <= bd1);
             }
         }
-        if (sel) {
-#pragma unroll
-            for (int f = 0; f < kFaces; ++f) {
-                inbox[b * kFaces + f] = dty ? fresh[b * kFaces + f] : 0ull;
-                if (dty)
-                    fresh[b * kFaces + f] = 0ull;
-            }
-            if (dty)
-                dirty[b] = 0u;
-        }
+        if (dty)
+            dirty[b] = 0u;
         const unsigned ball = __ballot_sync(0xffffffffu, sel);
         if (ball == 0u)
             continue;
@@ -1907,13 +1112,11 @@ __global__ void k_reset_control(Control *c, unsigned long long wait_ns, int hold
     c->dirty_count = 0u;
     c->n_list[0] = c->n_list[1] = 0u;
     c->work[0] = c->work[1] = 0u;
-    c->q_head = c->q_tail = 0ull;
-    c->pending = 0;
+    reset_queue(c);
     c->done = 0;
     c->error = 0;
     c->restart = 0;
     c->host_restart = 0;
-    c->epoch = 0;
 }
 
 // Brick layout -> the caller's x-fastest arrays (signed psi, public tags);
@@ -2029,9 +1232,7 @@ __global__ void k_set_bound(Control *c, double b0, double b1)
     c->bound[0] = b0;
     c->bound[1] = b1;
     c->done = 0;
-    c->q_head = 0ull;
-    c->q_tail = 0ull;
-    c->pending = 0;
+    reset_queue(c);
     c->minbits[0] = c->minbits[1] = 0x7ff0000000000000ull;
     c->dirty_count = 0u;
 }
@@ -2187,7 +1388,7 @@ int grid_for(long long n, int threads, int cap)
 }
 
 template <typename real, bool kTape>
-size_t march_smem() { return sizeof(WarpTile<real, kTape>) * kMarchWarps; }
+size_t march_smem() { return sizeof(MarchSmem<real, kTape>); }
 
 // Deterministic mode: face f of brick b is its boundary layer on side f
 // (0..5 = -x, +x, -y, +y, -z, +z), cell q = u + 8 v in the in-face
@@ -2275,6 +1476,26 @@ void with_flags(bool het, bool tape, bool aniso, Fn &&f)
     }
 }
 
+// One launch of the queue march (all: a restart with a fixed bound).
+template <typename real>
+void queue_march(const Geom &g, const DeviceState &s, const SolveParams &p, bool all, cudaStream_t st)
+{
+    // with no band width and a whole-brick look-ahead no cell is ever above a
+    // march's bound
+    const bool bounded = std::isfinite(p.width) || std::isfinite(p.ahead);
+    with_flags(s.spd != nullptr, s.tape != nullptr, p.aniso != 0, [&](auto H, auto P, auto A) {
+        constexpr bool h = decltype(H)::value, t = decltype(P)::value, an = decltype(A)::value;
+        const size_t sm = march_smem<real, t>();
+        const int ctas = s.march_ctas, th = kMarchWarps * 32;
+        if (all)
+            k_march_queue<real, h, t, an, true, true><<<ctas, th, sm, st>>>(g, s, p, p.spd_term);
+        else if (bounded)
+            k_march_queue<real, h, t, an, true, false><<<ctas, th, sm, st>>>(g, s, p, p.spd_term);
+        else
+            k_march_queue<real, h, t, an, false, false><<<ctas, th, sm, st>>>(g, s, p, p.spd_term);
+    });
+}
+
 template <typename real>
 cudaError_t restart_impl(const Geom &g, const DeviceState &s, const SolveParams &p,
                          cudaStream_t st, cudaEvent_t *ev, int *trace)
@@ -2282,22 +1503,16 @@ cudaError_t restart_impl(const Geom &g, const DeviceState &s, const SolveParams 
     const int rb = grid_for(g.nbricks, 256, 4096);
     const bool het = s.spd != nullptr, tape = s.tape != nullptr;
     const double sct = p.spd_term;
-    k_reduce<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.inmin, s.dirty, s.ctrl);
+    k_reduce<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.work, s.dirty, s.ctrl);
     k_control<<<1, 1, 0, st>>>(s.ctrl, p.width, p.stride, p.max_restarts);
     if (one_launch_schedule(p.schedule)) {
-        k_seed<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.inmin, s.ctrl, s.queued, s.queue);
+        const bool all = p.schedule == kSchedulePersistent;
+        k_seed<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.ctrl, s.work, s.queue, s.waiting, p.width, all);
         if (trace)
             k_trace_seed<<<1, 1, 0, st>>>(s.ctrl, trace);
         if (ev)
             cudaEventRecord(ev[0], st);
-        with_flags(het, tape, p.aniso != 0, [&](auto H, auto P, auto A) {
-            constexpr bool h = decltype(H)::value, t = decltype(P)::value, an = decltype(A)::value;
-            const size_t sm = march_smem<real, t>();
-            if (p.schedule == kScheduleContinuous)
-                k_march_continuous<real, h, t, an><<<s.march_ctas, kMarchWarps * 32, sm, st>>>(g, s, p, sct);
-            else
-                k_march_persistent<real, h, t, an><<<s.march_ctas, kMarchWarps * 32, sm, st>>>(g, s, p, sct);
-        });
+        queue_march<real>(g, s, p, all, st);
         if (ev)
             cudaEventRecord(ev[1], st);
         return cudaGetLastError();
@@ -2306,8 +1521,7 @@ cudaError_t restart_impl(const Geom &g, const DeviceState &s, const SolveParams 
         const int which = pass == 0 ? 0 : 1;
         if (pass >= 2)
             k_reset_list<<<1, 1, 0, st>>>(s.ctrl, 1);
-        k_select<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.dirty, s.fresh, s.inbox,
-                                           s.ctrl, s.list[which], which);
+        k_select<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.dirty, s.ctrl, s.list[which], which);
         if (trace)
             k_trace<<<1, 1, 0, st>>>(s.ctrl, which, pass, trace + 3 * pass);
         if (ev)
@@ -2354,12 +1568,16 @@ int configure_march(bool tape)
             const int sm = (int)march_smem<real, tt>();
             cudaFuncSetAttribute(k_march<real, hh, 1, tt, an>, attr, sm);
             cudaFuncSetAttribute(k_march<real, hh, 0, tt, an>, attr, sm);
-            cudaFuncSetAttribute(k_march_persistent<real, hh, tt, an>, attr, sm);
-            cudaFuncSetAttribute(k_march_continuous<real, hh, tt, an>, attr, sm);
+            cudaFuncSetAttribute(k_march_queue<real, hh, tt, an, true, true>, attr, sm);
+            cudaFuncSetAttribute(k_march_queue<real, hh, tt, an, true, false>, attr, sm);
+            cudaFuncSetAttribute(k_march_queue<real, hh, tt, an, false, false>, attr, sm);
             if (tt != tape)
                 return;
             int k = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_march_continuous<real, hh, tt, an>,
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_march_queue<real, hh, tt, an, false, false>,
+                                                          kMarchWarps * 32, sm);
+            n = k < n ? k : n;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_march_queue<real, hh, tt, an, true, false>,
                                                           kMarchWarps * 32, sm);
             n = k < n ? k : n;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_march<real, hh, 1, tt, an>, kMarchWarps * 32,
@@ -2486,21 +1704,13 @@ cudaError_t launch_march_to(int dtype, const Geom &g, const DeviceState &s, cons
 {
     k_set_bound<<<1, 1, 0, st>>>(s.ctrl, b0, b1);
     const int rb = grid_for(g.nbricks, 256, 4096);
-    const bool het = s.spd != nullptr, tape = s.tape != nullptr;
     if (dtype == 1) {
-        k_seed<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.inmin, s.ctrl, s.queued, s.queue);
-        with_flags(het, tape, p.aniso != 0, [&](auto H, auto P, auto A) {
-            k_march_persistent<double, decltype(H)::value, decltype(P)::value, decltype(A)::value>
-                <<<s.march_ctas, kMarchWarps * 32, march_smem<double, decltype(P)::value>(), st>>>(g, s, p,
-                                                                                                   p.spd_term);
-        });
+        k_seed<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.ctrl, s.work, s.queue, s.waiting, p.width,
+                                           true);
+        queue_march<double>(g, s, p, true, st);
     } else {
-        k_seed<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.inmin, s.ctrl, s.queued, s.queue);
-        with_flags(het, tape, p.aniso != 0, [&](auto H, auto P, auto A) {
-            k_march_persistent<float, decltype(H)::value, decltype(P)::value, decltype(A)::value>
-                <<<s.march_ctas, kMarchWarps * 32, march_smem<float, decltype(P)::value>(), st>>>(g, s, p,
-                                                                                                  p.spd_term);
-        });
+        k_seed<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.ctrl, s.work, s.queue, s.waiting, p.width, true);
+        queue_march<float>(g, s, p, true, st);
     }
     return cudaGetLastError();
 }
@@ -2512,9 +1722,9 @@ cudaError_t launch_minima(int dtype, const Geom &g, const DeviceState &s, cudaSt
     k_set_bound<<<1, 1, 0, st>>>(s.ctrl, 0.0, 0.0);
     const int rb = grid_for(g.nbricks, 256, 4096);
     if (dtype == 1)
-        k_reduce<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.inmin, s.dirty, s.ctrl);
+        k_reduce<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.work, s.dirty, s.ctrl);
     else
-        k_reduce<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.inmin, s.dirty, s.ctrl);
+        k_reduce<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.work, s.dirty, s.ctrl);
     return cudaGetLastError();
 }
 
@@ -2523,11 +1733,9 @@ cudaError_t launch_select(int dtype, const Geom &g, const DeviceState &s, int wh
 {
     const int rb = grid_for(g.nbricks, 256, 4096);
     if (dtype == 1)
-        k_select<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.dirty, s.fresh, s.inbox,
-                                             s.ctrl, s.list[which], which);
+        k_select<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.dirty, s.ctrl, s.list[which], which);
     else
-        k_select<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.dirty, s.fresh, s.inbox,
-                                            s.ctrl, s.list[which], which);
+        k_select<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.dirty, s.ctrl, s.list[which], which);
     return cudaGetLastError();
 }
 
@@ -2600,3 +1808,4 @@ int march_blocks_per_sm(int dtype, bool tape)
 }
 
 }  // namespace fmmgb
+

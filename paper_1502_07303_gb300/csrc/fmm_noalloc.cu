@@ -49,10 +49,9 @@ constexpr size_t kOffT = 0;
 constexpr size_t kOffTag = align256(kOffT + kCells * sizeof(double));
 constexpr size_t kOffBdelta = align256(kOffTag + kCells);
 constexpr size_t kOffBmin = align256(kOffBdelta + kNoAllocMaxBricks * sizeof(double));
-constexpr size_t kOffFresh = align256(kOffBmin + 2 * kNoAllocMaxBricks * sizeof(double));
-constexpr size_t kOffInmin = align256(kOffFresh + kFaces * kNoAllocMaxBricks * sizeof(unsigned long long));
-constexpr size_t kOffInbox = align256(kOffInmin + 2 * kNoAllocMaxBricks * sizeof(unsigned long long));
-constexpr size_t kOffDirty = align256(kOffInbox + kFaces * kNoAllocMaxBricks * sizeof(unsigned long long));
+constexpr size_t kOffWork = align256(kOffBmin + 2 * kNoAllocMaxBricks * sizeof(double));
+constexpr size_t kOffWaiting = align256(kOffWork + kNoAllocMaxBricks * sizeof(unsigned long long));
+constexpr size_t kOffDirty = align256(kOffWaiting + kNoAllocMaxBricks * sizeof(unsigned long long));
 constexpr size_t kOffList0 = align256(kOffDirty + kNoAllocMaxBricks * sizeof(unsigned));
 constexpr size_t kOffList1 = align256(kOffList0 + kNoAllocMaxBricks * sizeof(int));
 constexpr size_t kOffQueue = align256(kOffList1 + kNoAllocMaxBricks * sizeof(int));
@@ -168,9 +167,8 @@ extern "C" fmm_status fmm_reinit_signed_distance_noalloc(const fmm_config *cfg, 
     s.tag = base + kOffTag;
     s.bdelta = base + kOffBdelta;
     s.bmin = base + kOffBmin;
-    s.fresh = (unsigned long long *)(base + kOffFresh);
-    s.inmin = (unsigned long long *)(base + kOffInmin);
-    s.inbox = (unsigned long long *)(base + kOffInbox);
+    s.work = (unsigned long long *)(base + kOffWork);
+    s.waiting = (unsigned long long *)(base + kOffWaiting);
     s.dirty = (unsigned *)(base + kOffDirty);
     s.list[0] = (int *)(base + kOffList0);
     s.list[1] = (int *)(base + kOffList1);
@@ -180,7 +178,7 @@ extern "C" fmm_status fmm_reinit_signed_distance_noalloc(const fmm_config *cfg, 
     s.spd = nullptr;
     s.tape = nullptr;
     const int per_sm = march_blocks_per_sm(cfg->dtype, false);
-    s.march_ctas = cfg->ctas > 0 ? cfg->ctas : sms * per_sm;
+    s.march_ctas = cfg->ctas > 0 ? cfg->ctas : march_grid(sms * per_sm, g.nbricks);
 
     SolveParams p;
     memset(&p, 0, sizeof(p));
@@ -217,8 +215,8 @@ extern "C" fmm_status fmm_reinit_signed_distance_noalloc(const fmm_config *cfg, 
     } while (0)
     // clear what the solve reads before it writes
     NA_CUDA(launch_reset_control(s, st, p.wait_ns, p.hold));
-    NA_CUDA(cudaMemsetAsync(s.fresh, 0, (size_t)g.nbricks * kFaces * sizeof(unsigned long long), st));
-    NA_CUDA(cudaMemsetAsync(s.inmin, 0xff, (size_t)g.nbricks * 2 * sizeof(unsigned long long), st));
+    NA_CUDA(cudaMemsetAsync(s.work, 0xff, (size_t)g.nbricks * sizeof(unsigned long long), st));
+    NA_CUDA(cudaMemsetAsync(s.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
     NA_CUDA(cudaMemsetAsync(s.dirty, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     NA_CUDA(cudaMemsetAsync(s.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
     NA_CUDA(cudaMemsetAsync(s.queued, 0, (size_t)g.nbricks * sizeof(unsigned), st));

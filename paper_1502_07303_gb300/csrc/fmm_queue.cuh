@@ -25,6 +25,11 @@ __device__ __forceinline__ unsigned long long vload(const unsigned long long *p)
 }
 __device__ __forceinline__ int vload(const int *p) { return *(const volatile int *)p; }
 
+// Order this thread's earlier memory operations before its later ones for a
+// reader that does the same (message passing).  Store-then-load checks on two
+// words need the stronger __threadfence().
+__device__ __forceinline__ void fence_acq_rel() { asm volatile("fence.acq_rel.gpu;" ::: "memory"); }
+
 // Push brick b (the caller has claimed queued[b] and counted it in pending).
 __device__ __forceinline__ bool queue_push(Control *c, unsigned long long *q, unsigned long long cap,
                                            long long b)

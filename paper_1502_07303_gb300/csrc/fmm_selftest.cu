@@ -40,7 +40,7 @@ extern "C" fmm_status fmm_selftest_fp64(const double *a, const double *b, double
 }
 
 // ---------------------------------------------------------------------------
-// The double-grid root of Algorithm 11 (fmm_df.cuh's df_shifted_root) on
+// The double-grid root of Algorithm 11 (fmm_df.cuh's df_root) on
 // caller arrays: sorted upwind values m <= v1 <= v2 (nd of them used), speed
 // term q; returns the root and the size of the causal set it chose.
 // ---------------------------------------------------------------------------
@@ -55,7 +55,9 @@ __global__ void k_selftest_root(const double *__restrict__ m, const double *__re
          i += (long long)gridDim.x * blockDim.x) {
         double t = 0.0;
         // as the march computes it when it records the upwind sets
-        const int k = fmmgb::df_shifted_root<true>(m[i], v1[i], v2[i], nd[i], q[i], t);
+        const double inf = __longlong_as_double(0x7ff0000000000000ll);
+        const int k = fmmgb::df_root<true>(m[i], nd[i] >= 2 ? v1[i] : inf, nd[i] >= 3 ? v2[i] : inf,
+                                             fmmgb::df_speed(q[i]), q[i], t);
         t_out[i] = k ? t : __longlong_as_double(0x7ff0000000000000ll);
         k_out[i] = k;
     }
