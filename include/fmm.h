@@ -110,7 +110,7 @@ typedef struct {
                               bucket of each side's minimum over the whole
                               grid and re-solves their neighbours (Jacobi
                               within the step, corrections as in the brick
-                              march), three grid-wide launches per step; no
+                              march), up to 256 steps per launch; no
                               tape, no resume (max_restarts limits the
                               steps); the schedule of the second-order march
                               and, in first order, the same solution as the

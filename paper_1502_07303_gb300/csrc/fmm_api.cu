@@ -438,9 +438,9 @@ fmm_status run_restarts(fmm_handle *hd, void *T_out, uint8_t *tags_out, long lon
 }
 
 // The cell-parallel march (schedule 4): Algorithm 9, then bucket steps until
-// the step that finds no BAND cell at or below width_band, enqueued in
-// growing batches with the termination flag read between batches (steps
-// enqueued after it return at once); then the output conversion.  The march
+// the step that finds no BAND cell at or below width_band, run in
+// launches of growing length with the termination flag read between them (a
+// launch ends at that step); then the output conversion.  The march
 // has no restart boundary to stop on: a solve stopped by max_restarts (here
 // a limit on the bucket steps) or timeout_s cannot be resumed.
 fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
@@ -457,7 +457,7 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
     if (!hd->cell_next)
         FMM_CUDA(hd, alloc(&hd->cell_next, cells * hd->rsize));
     if (!hd->cell_min)
-        FMM_CUDA(hd, alloc(&hd->cell_min, 4 * sizeof(unsigned long long)));
+        FMM_CUDA(hd, alloc(&hd->cell_min, 5 * sizeof(unsigned long long)));
     const bool timing = hd->cfg.time_kernels != 0;
     while (timing && hd->events.size() < 2) {
         cudaEvent_t e;
@@ -468,7 +468,7 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
     if (timing)
         FMM_CUDA(hd, cudaEventRecord(hd->events[0], st));
     FMM_CUDA(hd, launch_cell_begin(dt, g, s, p, hd->cell_next, hd->cell_min, st));
-    long long launches = 4;   // control reset; seed, relax, apply
+    long long launches = 5;   // control reset; seed, relax, apply, brick minima
     const auto t0 = std::chrono::steady_clock::now();
     const double limit_s = hd->cfg.timeout_s > 0 ? (double)hd->cfg.timeout_s : 600.0;
     bool timed_out = false, limited = false;
@@ -477,13 +477,12 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
         long long n = batch;
         if (p.max_restarts > 0 && step + n > p.max_restarts)
             n = p.max_restarts - step;
-        for (long long r = 0; r < n; ++r, ++step) {
-            FMM_CUDA(hd, launch_cell_step(dt, g, s, p, hd->cell_next, hd->cell_min, step, st));
-            launches += 3;
-        }
+        FMM_CUDA(hd, launch_cell_steps(dt, g, s, p, hd->cell_next, hd->cell_min, step, (int)n, st));
+        launches += 1;
+        step += n;
         FMM_CUDA(hd, cudaMemcpyAsync(hd->h_ctrl, s.ctrl, sizeof(Control), cudaMemcpyDeviceToHost, st));
         FMM_CUDA(hd, cudaStreamSynchronize(st));
-        if (hd->h_ctrl->done)
+        if (hd->h_ctrl->done || (hd->h_ctrl->error & ERR_SPIN))
             break;
         if (p.max_restarts > 0 && step >= p.max_restarts) {
             limited = true;
@@ -493,11 +492,12 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
             timed_out = true;
             break;
         }
-        if (batch < 64)
+        if (batch < 256)
             batch *= 2;
     }
     if (timing)
         FMM_CUDA(hd, cudaEventRecord(hd->events[1], st));
+    const long long march_launches = launches - 1;
     const Control c = *hd->h_ctrl;
     {
         const fmm_status r = write_outputs(hd, T_out, tags_out, launches);
@@ -511,7 +511,7 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
     hd->stats.n_bricks = g.nbricks;
     hd->stats.error_flags = c.error;
     hd->stats.kernel_launches = launches + hd->pre_launches;
-    hd->stats.march_launches = 3 * (step + 1);
+    hd->stats.march_launches = march_launches;
     hd->pre_launches = 0;
     hd->trace.clear();
     if (timing) {
@@ -524,6 +524,8 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
     hd->fwd_ctrl = c;
     if (timed_out)
         return fail(hd, FMM_ERR_TIMEOUT, "the solve exceeded its wall-clock limit (timeout_s)");
+    if (c.error & ERR_SPIN)
+        return fail(hd, FMM_ERR_TIMEOUT, "a bounded wait of the cell-parallel march gave up");
     if (limited)
         return fail(hd, FMM_ERR_TIMEOUT, "the step limit (max_restarts) was reached before termination");
     return FMM_OK;

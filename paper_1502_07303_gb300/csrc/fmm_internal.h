@@ -296,12 +296,14 @@ cudaError_t launch_reset_list(const DeviceState &s, int which, cudaStream_t stre
 cudaError_t launch_init_fixed(int dtype, const Geom &g, const DeviceState &s, const void *T0,
                               cudaStream_t stream);
 // next: one value per brick-layout cell (the step's new values); mins: 4
-// words (two slots of the per-side BAND minima).  begin runs Algorithm 9 and
-// fills slot 0; step k accepts from slot k & 1 and fills the other one.
+// words (two slots of the per-side BAND minima) and a fifth for the grid
+// barrier.  begin runs Algorithm 9 and fills slot 0; step k accepts from slot
+// k & 1 and fills the other one.
 cudaError_t launch_cell_begin(int dtype, const Geom &g, const DeviceState &s, const SolveParams &p,
                               void *next, unsigned long long *mins, cudaStream_t stream);
-cudaError_t launch_cell_step(int dtype, const Geom &g, const DeviceState &s, const SolveParams &p,
-                             void *next, unsigned long long *mins, long long step, cudaStream_t stream);
+// steps step .. step + n - 1 in one launch (ends early when the march is done)
+cudaError_t launch_cell_steps(int dtype, const Geom &g, const DeviceState &s, const SolveParams &p,
+                              void *next, unsigned long long *mins, long long step, int n, cudaStream_t stream);
 
 // Adjoint (fmm_adjoint.cu).  The reverse sweep can run by levels of |psi|
 // of kAdjointLevelStep h each (at most kAdjointMaxLevels); 0 (the default)
