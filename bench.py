@@ -387,27 +387,15 @@ def measure_e2e(fmm, torch, phi_host, p, dtype, steps, warmup, stream, params):
     return statistics.mean(times), nbytes, T_host.numel() * T_host.element_size()
 
 
-# bytes one bucket step of the cell-parallel march streams per cell (brick
-# layout, fp64): accept reads psi + tag (9), relax reads psi + tag (9; the
-# neighbours' values come from L1/L2), apply reads psi + tag + the new-value
-# buffer (17)
-CELL_STEP_BYTES = {"f64": 35, "f32": 19}
-
-
 def measure_second_order(fmm, torch, wl, stream, flush, n=256, steps=3, warmup=2):
     """The cell-parallel march (schedule 4) in first and second order on the
     single-sphere reinitialisation (fp64), with the error of each against
     the exact signed distance (phi0 is exact for one sphere), and the brick
-    march (first order, library defaults) on the same workload for scale.
-    Roofline: the bytes the march's grid-wide passes stream per bucket step
-    (CELL_STEP_BYTES per brick-layout cell) over the device time of the
-    march, against the measured copy peak."""
+    march (first order, library defaults) on the same workload for scale."""
     p = wl.single_sphere(n=n, radius=RADIUS, device="cuda")
     phi = p.phi0.contiguous()
     exact = phi.abs()
     out = {"workload": f"reinit single sphere r={RADIUS} centred, {n}^3, fp64", "points": p.n_points}
-    cells = ((n + 7) // 8) ** 3 * 512
-    peak, peak_kind = peaks()
     for name, prm in (("brick_first_order", {}), ("cell_first_order", {"schedule": 4}),
                       ("cell_second_order", {"schedule": 4, "accuracy": 2})):
         r = measure(fmm, torch, p, torch.float64, steps, warmup, flush, stream, prm, phi=phi)
@@ -419,15 +407,13 @@ def measure_second_order(fmm, torch, wl, stream, flush, n=256, steps=3, warmup=2
                "accepted_per_point": r["stats"]["accepted"] / p.n_points}
         if prm.get("schedule") == 4:
             # bucket steps that accepted cells, plus the one that ended the
-            # march (steps enqueued after it return at once)
+            # march; a step visits the bricks at the front only, so its cost
+            # is a time per step and no share of the HBM rate
             nsteps = r["stats"]["restarts"] + 1
-            achieved = CELL_STEP_BYTES["f64"] * cells * nsteps / (r["march_ms"] / 1e3) / 1e9
             rec["bucket_steps"] = nsteps
-            rec["roofline"] = {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
-                               "frac": achieved / peak, "peak_kind": peak_kind,
-                               "bytes_per_cell_per_step": CELL_STEP_BYTES["f64"],
-                               "kernels": "k_cell_accept + k_cell_relax + k_cell_apply",
-                               "march_ms": r["march_ms"], "share_of_step": r["march_ms"] / r["ms"]}
+            rec["kernels"] = "k_cell_steps"
+            rec["march_ms"] = r["march_ms"]
+            rec["us_per_step"] = r["march_ms"] * 1e3 / nsteps
         out[name] = rec
         del T, err
     out["second_vs_first_order_err_mean"] = out["cell_first_order"]["err_mean"] / out["cell_second_order"]["err_mean"]
@@ -590,6 +576,8 @@ def roofline_alu(r, pts, kernel, dt, workload, fp64_peak, sms, sm_mhz):
 
 
 def kernel_name(params):
+    """The march of a schedule as the profile records name it (the continuous
+    and the persistent one are k_march_queue)."""
     return {1: "k_march", 2: "k_march_persistent"}.get(params.get("schedule", 0), "k_march_continuous")
 
 
