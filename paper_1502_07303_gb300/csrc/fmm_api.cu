@@ -266,7 +266,7 @@ fmm_status run_solve(fmm_handle *hd, void *T_out, uint8_t *tags_out)
     FMM_CUDA(hd, cudaMemsetAsync(s.work, 0xff, (size_t)g.nbricks * sizeof(unsigned long long), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.dirty, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
-    FMM_CUDA(hd, cudaMemsetAsync(s.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
+    FMM_CUDA(hd, cudaMemsetAsync(s.waiting, 0, waiting_bytes(g.nbricks), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queued, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, launch_front_init(dt, g, s, hd->params, st));
     return run_restarts(hd, T_out, tags_out, 2);   // control reset, front init
@@ -711,7 +711,7 @@ fmm_status fmm_create(const fmm_config *cfg, const void *speed, double speed_con
     ALLOC(s.bdelta, nb * hd->rsize);
     ALLOC(s.bmin, 2 * nb * hd->rsize);
     ALLOC(s.work, nb * sizeof(unsigned long long));
-    ALLOC(s.waiting, nb * sizeof(unsigned long long));
+    ALLOC(s.waiting, waiting_bytes(g.nbricks));
     ALLOC(s.dirty, nb * sizeof(unsigned));
     ALLOC(s.list[0], nb * sizeof(int));
     ALLOC(s.list[1], nb * sizeof(int));
@@ -910,7 +910,7 @@ fmm_status fmm_resume(fmm_handle *hd, int64_t more_restarts, void *T_out, uint8_
                                     hd->stream);
     // (a launch stopped by its restart limit leaves entries in the waiting ring)
     if (e == cudaSuccess)
-        e = cudaMemsetAsync(hd->st.waiting, 0, (size_t)hd->geom.nbricks * sizeof(unsigned long long), hd->stream);
+        e = cudaMemsetAsync(hd->st.waiting, 0, waiting_bytes(hd->geom.nbricks), hd->stream);
     if (e == cudaSuccess && hd->st.faces)
         e = launch_faces_build(hd->cfg.dtype, hd->geom, hd->st, hd->stream);   // from the stopped state
     if (e != cudaSuccess) {
@@ -979,7 +979,7 @@ fmm_status fmm_dd_start(fmm_handle *hd, const void *phi0, int64_t extra_lo, int6
     FMM_CUDA(hd, cudaMemsetAsync(s.work, 0xff, (size_t)g.nbricks * sizeof(unsigned long long), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.dirty, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
-    FMM_CUDA(hd, cudaMemsetAsync(s.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
+    FMM_CUDA(hd, cudaMemsetAsync(s.waiting, 0, waiting_bytes(g.nbricks), st));
     FMM_CUDA(hd, cudaMemsetAsync(s.queued, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     FMM_CUDA(hd, launch_front_init(dt, g, s, hd->params, st));
     FMM_CUDA(hd, cudaStreamSynchronize(st));
@@ -1187,7 +1187,7 @@ fmm_status fmm_checkpoint_load(fmm_handle *hd, const void *host_buf, int64_t siz
     // the queue is empty between restarts
     const Geom &g = hd->geom;
     FMM_CUDA(hd, cudaMemset(hd->st.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long)));
-    FMM_CUDA(hd, cudaMemset(hd->st.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long)));
+    FMM_CUDA(hd, cudaMemset(hd->st.waiting, 0, waiting_bytes(g.nbricks)));
     FMM_CUDA(hd, cudaMemset(hd->st.queued, 0, (size_t)g.nbricks * sizeof(unsigned)));
     hd->complete = hdr.complete != 0;
     hd->resumable = hdr.resumable != 0;
@@ -1322,7 +1322,7 @@ fmm_status fmm_create_batch(int n_grids, const int64_t *dims, const double *h,
     ALLOC(s.bdelta, nb * hd->rsize);
     ALLOC(s.bmin, 2 * nb * hd->rsize);
     ALLOC(s.work, nb * sizeof(unsigned long long));
-    ALLOC(s.waiting, nb * sizeof(unsigned long long));
+    ALLOC(s.waiting, waiting_bytes(g.nbricks));
     ALLOC(s.dirty, nb * sizeof(unsigned));
     ALLOC(s.list[0], nb * sizeof(int));
     ALLOC(s.list[1], nb * sizeof(int));

@@ -6,6 +6,8 @@
 #include <cstdint>
 #include <cuda_runtime.h>
 
+#include "fmm_ring.h"
+
 namespace fmmgb {
 
 // ---------------------------------------------------------------------------
@@ -145,6 +147,8 @@ constexpr int kSchedulePhased = 1;
 constexpr int kSchedulePersistent = 2;
 constexpr int kScheduleContinuous = 3;
 constexpr int kScheduleCell = 4;     // cell-parallel bucketed march (fmm_cell.cu)
+// bytes of the waiting ring
+inline size_t waiting_bytes(long long nbricks) { return (size_t)waiting_slots(nbricks) * sizeof(unsigned long long); }
 constexpr int kMarchWarps = 4;   // bricks in flight per CTA of the march kernels
 // Continuous schedule: the bound rises once fewer bricks than this are queued
 // or marching: the warps of the march launch (half of them left 30% of the
@@ -199,7 +203,7 @@ struct DeviceState {
     unsigned long long *work;    // 1 per brick: smallest work it has, as float
                                  // bits (rounded down; >= the bits of +inf:
                                  // none), << 32 | flags (kWorkActive, kWorkWaiting)
-    unsigned long long *waiting; // waiting ring, laid out as the queue
+    unsigned long long *waiting; // waiting ring, entries as in the queue: waiting_slots() of them
     void *faces;        // deterministic mode, 6 x 64 per brick: its boundary
                         // layers (known value or +inf) as of the last pass
     unsigned int *dirty;         // 1 per brick: has pending overlap changes

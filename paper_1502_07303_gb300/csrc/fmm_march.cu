@@ -448,7 +448,9 @@ __device__ __forceinline__ unsigned long long vloadu(const unsigned long long *p
     return *(const volatile unsigned long long *)p;
 }
 
-// Put brick b into ring slot t (waits, bounded, for a slot still being read).
+// Put brick b at position t of the ready queue or the waiting ring (waits,
+// bounded, for a queue slot still being read; the waiting ring has a free slot
+// for every append, fmm_ring.h).
 __device__ __forceinline__ void ring_put(Control *c, unsigned long long *q, unsigned long long cap,
                                          unsigned long long t, long long b)
 {
@@ -594,7 +596,7 @@ __device__ __forceinline__ void finish_brick(const DeviceState &s, unsigned long
         if (act == 1)
             ring_put(c, s.queue, cap, tq + __popc(bq & below), tb);
         else if (act == 2)
-            ring_put(c, s.waiting, cap, tw + __popc(bw & below), tb);
+            ring_put(c, s.waiting, waiting_slots((long long)cap), tw + __popc(bw & below), tb);
     }
     __syncwarp();
 }
@@ -846,7 +848,7 @@ __device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long l
 {
     Control *c = s.ctrl;
     const auto &lv = c->level[ep & 1];
-    const unsigned long long end = vloadu(&lv.end);
+    const unsigned long long end = vloadu(&lv.end), wcap = waiting_slots((long long)cap);
     const int chunk = vload(&lv.chunk);
     const float bound = *(const volatile float *)&lv.bound;
     const unsigned long long first = vloadu(&lv.base) + (unsigned long long)ch * (unsigned)chunk;
@@ -856,7 +858,7 @@ __device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long l
         long long b = -1;
         if (pos < end) {
             // the entry may still be on its way from the warp that counted it
-            unsigned long long *slot = s.waiting + pos % cap;
+            unsigned long long *slot = s.waiting + pos % wcap;
             const unsigned long long want = pos & 0xffffffffull;
             unsigned long long v = vloadu(slot);
             if (v == 0ull || (v >> 32) != want) {
@@ -913,7 +915,7 @@ __device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long l
         if (act == 1)
             ring_put(c, s.queue, cap, tq + __popc(bq & below), b);
         else if (act == 2)
-            ring_put(c, s.waiting, cap, tw + __popc(bw & below), b);
+            ring_put(c, s.waiting, wcap, tw + __popc(bw & below), b);
     }
     kept = __reduce_min_sync(FULL, kept);
     if (lane == 0) {

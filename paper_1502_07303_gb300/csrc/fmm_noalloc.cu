@@ -51,7 +51,7 @@ constexpr size_t kOffBdelta = align256(kOffTag + kCells);
 constexpr size_t kOffBmin = align256(kOffBdelta + kNoAllocMaxBricks * sizeof(double));
 constexpr size_t kOffWork = align256(kOffBmin + 2 * kNoAllocMaxBricks * sizeof(double));
 constexpr size_t kOffWaiting = align256(kOffWork + kNoAllocMaxBricks * sizeof(unsigned long long));
-constexpr size_t kOffDirty = align256(kOffWaiting + kNoAllocMaxBricks * sizeof(unsigned long long));
+constexpr size_t kOffDirty = align256(kOffWaiting + waiting_slots(kNoAllocMaxBricks) * sizeof(unsigned long long));
 constexpr size_t kOffList0 = align256(kOffDirty + kNoAllocMaxBricks * sizeof(unsigned));
 constexpr size_t kOffList1 = align256(kOffList0 + kNoAllocMaxBricks * sizeof(int));
 constexpr size_t kOffQueue = align256(kOffList1 + kNoAllocMaxBricks * sizeof(int));
@@ -216,7 +216,7 @@ extern "C" fmm_status fmm_reinit_signed_distance_noalloc(const fmm_config *cfg, 
     // clear what the solve reads before it writes
     NA_CUDA(launch_reset_control(s, st, p.wait_ns, p.hold));
     NA_CUDA(cudaMemsetAsync(s.work, 0xff, (size_t)g.nbricks * sizeof(unsigned long long), st));
-    NA_CUDA(cudaMemsetAsync(s.waiting, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
+    NA_CUDA(cudaMemsetAsync(s.waiting, 0, waiting_bytes(g.nbricks), st));
     NA_CUDA(cudaMemsetAsync(s.dirty, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     NA_CUDA(cudaMemsetAsync(s.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
     NA_CUDA(cudaMemsetAsync(s.queued, 0, (size_t)g.nbricks * sizeof(unsigned), st));

@@ -1,0 +1,42 @@
+"""The protocol of the one-launch brick scheduler as a host model
+(tests/host/scheduler_model.cpp: warps take turns at random, one atomic
+operation a turn) with the ring sizes of csrc/fmm_ring.h: it must always end."""
+import os
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+SEEDS = 20
+
+
+@pytest.fixture(scope="module")
+def model(tmp_path_factory):
+    exe = str(tmp_path_factory.mktemp("model") / "scheduler_model")
+    subprocess.run(["g++", "-O2", "-std=c++17", "-Wall", "-I",
+                    os.path.join(ROOT, "paper_1502_07303_gb300", "csrc"),
+                    os.path.join(ROOT, "tests", "host", "scheduler_model.cpp"), "-o", exe], check=True)
+
+    def run(bricks, waiting, warps, levels=40, release=1, slots=0):
+        args = (bricks, waiting, warps, levels, release, SEEDS, slots)
+        r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=300)
+        return r.returncode, r.stdout
+    return run
+
+
+# bricks, bricks that wait, warps: chunks of a scan of one and of many warp
+# loads, half of the bricks waiting and all of them
+GRIDS = [(1, 1, 4), (33, 33, 4), (64, 64, 4), (512, 400, 4), (512, 512, 4), (1000, 800, 12),
+         (4096, 2600, 32), (4096, 4096, 32)]
+
+
+@pytest.mark.parametrize("bricks,waiting,warps", GRIDS)
+def test_appends_never_wait_for_the_scan(model, bricks, waiting, warps):
+    rc, out = model(bricks, waiting, warps)
+    assert rc == 0, out
+
+
+def test_one_slot_per_brick_would_stall(model):
+    """The model does find a ring that is too small."""
+    rc, out = model(512, 512, 4, slots=512)
+    assert rc == 2, out
