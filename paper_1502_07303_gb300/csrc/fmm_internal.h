@@ -77,9 +77,9 @@ struct Control {
     unsigned long long w_head;       // waiting ring: entries below are scanned or being scanned
     struct {
         unsigned long long base, end;   // ring positions of the scan
-        int nchunks, chunk;
+        unsigned long long chunks;      // raise number << 32 | chunks of the scan (chunk_word)
+        int chunk;                      // ring entries of a chunk
         float bound;                    // marches start at or below it
-        int pad;
     } level[2];
     int scan_done;                   // chunks of the scan that are done
     unsigned scan_min;               // smallest value it kept waiting (float bits)

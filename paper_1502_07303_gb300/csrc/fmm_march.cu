@@ -715,13 +715,13 @@ __device__ bool try_raise(Control *c, const SolveParams &p, int pend)
     const unsigned long long w = vloadu(&c->scan_word);
     const int ep = (int)(w >> 32);
     const auto *lv = &c->level[ep & 1];
-    if (vload(&c->scan_done) < vload(&lv->nchunks) || vloadu(&c->w_tail) == vloadu(&c->w_head))
+    if (vload(&c->scan_done) < (int)(unsigned)vloadu(&lv->chunks) || vloadu(&c->w_tail) == vloadu(&c->w_head))
         return false;
     if (atomicCAS(&c->raise_lock, ep, ep + 1) != ep)
         return false;
     __threadfence();
     const unsigned long long base = vloadu(&c->w_head), end = vloadu(&c->w_tail);
-    bool ok = end != base && vload(&c->scan_done) >= vload(&lv->nchunks);
+    bool ok = end != base && vload(&c->scan_done) >= (int)(unsigned)vloadu(&lv->chunks);
     if (ok && p.max_restarts > 0 && (long long)vload(&c->restart) >= p.max_restarts) {
         // the restart limit counts the raises too
         atomicOr(&c->error, ERR_RESTARTS);
@@ -746,7 +746,7 @@ __device__ bool try_raise(Control *c, const SolveParams &p, int pend)
     *(volatile unsigned long long *)&nl->base = base;
     *(volatile unsigned long long *)&nl->end = end;
     *(volatile int *)&nl->chunk = chunk;
-    *(volatile int *)&nl->nchunks = (int)((count + chunk - 1) / chunk);
+    *(volatile unsigned long long *)&nl->chunks = chunk_word((unsigned)(ep + 1), (count + chunk - 1) / chunk);
     *(volatile float *)&nl->bound = nb;
     *(volatile unsigned long long *)&c->w_head = end;
     *(volatile int *)&c->scan_done = 0;
@@ -762,7 +762,7 @@ __device__ bool try_raise(Control *c, const SolveParams &p, int pend)
 __device__ bool launch_done(Control *c, bool limited)
 {
     const int ep = (int)(vloadu(&c->scan_word) >> 32);
-    if (vload(&c->scan_done) < vload(&c->level[ep & 1].nchunks))
+    if (vload(&c->scan_done) < (int)(unsigned)vloadu(&c->level[ep & 1].chunks))
         return false;
     __threadfence();
     if (vload(&c->pending) != 0)
@@ -772,7 +772,7 @@ __device__ bool launch_done(Control *c, bool limited)
         return false;
     __threadfence();
     return vload(&c->raise_lock) == ep && (int)(vloadu(&c->scan_word) >> 32) == ep &&
-           vload(&c->scan_done) >= vload(&c->level[ep & 1].nchunks);
+           vload(&c->scan_done) >= (int)(unsigned)vloadu(&c->level[ep & 1].chunks);
 }
 
 // One lane: the next job of the warp.  job 0: march brick arg; 1: scan chunk
@@ -808,13 +808,14 @@ __device__ void next_job(Control *c, unsigned long long *q, unsigned long long c
             const int pend = vload(&c->pending);
             unsigned long long w = vloadu(&c->scan_word);
             if (!kAll) {
-                if ((int)(unsigned)w < vload(&c->level[(w >> 32) & 1u].nchunks)) {
+                if (claimed_chunk(w, vloadu(&c->level[(w >> 32) & 1u].chunks)) >= 0) {
                     w = atomicAdd(&c->scan_word, 1ull);
                     __threadfence();   // the level this chunk belongs to
                     ep_out = (int)(w >> 32);
-                    if ((int)(unsigned)w < vload(&c->level[ep_out & 1].nchunks)) {
+                    const int ch = claimed_chunk(w, vloadu(&c->level[ep_out & 1].chunks));
+                    if (ch >= 0) {
                         job = 1;
-                        arg = (long long)(unsigned)w;
+                        arg = ch;
                         return;
                     }
                 }
@@ -873,7 +874,7 @@ __device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long l
                 }
             }
             if (v != 0ull && (v >> 32) == want) {
-                atomicExch(slot, 0ull);
+                v = atomicExch(slot, 0ull);
                 b = (long long)(v & 0xffffffffull) - 1;
             }
         }
@@ -997,7 +998,7 @@ __global__ void k_seed(Geom g, const real *__restrict__ bmin, Control *ctrl, uns
     if (blockIdx.x == 0 && threadIdx.x == 0) {
         // level 0: no scan, the bound of k_control
         ctrl->level[0].base = ctrl->level[0].end = 0ull;
-        ctrl->level[0].nchunks = 0;
+        ctrl->level[0].chunks = chunk_word(0, 0);
         ctrl->level[0].chunk = 32;
         ctrl->level[0].bound = bd;
         ctrl->scan_min = __float_as_uint(bd);

@@ -1,5 +1,6 @@
-// fmm_ring.h -- sizes of the brick scheduler's rings: plain C++, shared by the
-// kernels, the host code and a host model of the scheduler.
+// fmm_ring.h -- sizes of the brick scheduler's rings and the claim of a scan's
+// chunk: plain C++, shared by the kernels, the host code and a host model of the
+// scheduler.
 #pragma once
 
 #ifdef __CUDACC__
@@ -20,6 +21,21 @@ namespace fmmgb {
 FMM_HOST_DEVICE constexpr unsigned long long waiting_slots(long long nbricks)
 {
     return 2ull * (unsigned long long)nbricks;
+}
+
+// The chunks of a scan: raise number << 32 | count.  A claim is what the shared
+// counter (raise number << 32 | next chunk) held before it was advanced.  Its
+// chunk is the claimer's only if it belongs to that raise: a claim past the last
+// chunk holds nothing back, so two raises later the word may describe another
+// scan with more chunks.  Returns the chunk, or -1.  (A chunk that was claimed
+// keeps its scan open, so the word cannot change under a valid claim.)
+FMM_HOST_DEVICE constexpr unsigned long long chunk_word(unsigned raise, unsigned count)
+{
+    return ((unsigned long long)raise << 32) | count;
+}
+FMM_HOST_DEVICE constexpr int claimed_chunk(unsigned long long claim, unsigned long long chunks)
+{
+    return claim >> 32 == chunks >> 32 && (unsigned)claim < (unsigned)chunks ? (int)(unsigned)claim : -1;
 }
 
 }  // namespace fmmgb

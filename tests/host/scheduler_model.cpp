@@ -6,11 +6,11 @@
 // launch is done (exit 0), when no warp can move (stalled, exit 2), or when a
 // chunk of a scan is taken twice, an entry is lost or work is left (exit 3).
 //
-//   scheduler_model bricks waiting warps levels release seeds ring_slots
+//   scheduler_model bricks waiting warps levels release seeds ring_slots any_raise
 //
 // waiting: bricks that wait at the start, their work spread over `levels`
 // strides; release: strides a raise goes up; ring_slots: slots of the waiting
-// ring (0: the library's).
+// ring (0: the library's); any_raise: 1 takes a claim without a look at its raise.
 #include "fmm_ring.h"
 
 #include <algorithm>
@@ -34,7 +34,7 @@ struct Put {
 struct Level {
     u64 base = 0, end = 0;
     int chunk = 32;
-    unsigned nchunks = 0;
+    u64 chunks = 0;
     int bound = 0;
 };
 enum State { POLL, CLAIM, ACCEPT, READ, DECIDE, COUNT, PUTS, SCANNED, TAKE, MARCH, FLAG, COUNT2, PUTS2, STOP };
@@ -56,6 +56,7 @@ struct Model {
     int n, nw;
     u64 cap_w, cap_q;
     int stride, budget;
+    bool any_raise = false;
     std::mt19937_64 rng;
     std::vector<int> key, fl;
     std::vector<u64> queue, ring;
@@ -98,7 +99,7 @@ struct Model {
     {
         const int ep = (int)(scan_word >> 32);
         const Level &lv = level[ep & 1];
-        if (scan_done < (int)lv.nchunks || w_tail == w_head || raise_lock != ep)
+        if (scan_done < (int)(unsigned)lv.chunks || w_tail == w_head || raise_lock != ep)
             return false;
         Level &nl = level[(ep + 1) & 1];
         nl.base = w_head;
@@ -106,11 +107,12 @@ struct Model {
         nl.bound = std::max(lv.bound, scan_min == kNone ? lv.bound : scan_min) + stride;
         const unsigned count = (unsigned)(nl.end - nl.base);
         nl.chunk = (((int)((count + nw - 1) / nw)) + 31) & ~31;
-        nl.nchunks = (count + nl.chunk - 1) / nl.chunk;
+        const unsigned nchunks = (count + (unsigned)nl.chunk - 1) / (unsigned)nl.chunk;
+        nl.chunks = fmmgb::chunk_word((unsigned)(ep + 1), nchunks);
         w_head = nl.end;
         scan_done = 0;
         scan_min = kNone;
-        seen.assign(nl.nchunks, 0);
+        seen.assign(nchunks, 0);
         raise_lock = ep + 1;
         scan_word = (u64)(ep + 1) << 32;
         return true;
@@ -128,13 +130,13 @@ struct Model {
             return true;
         }
         const int ep = (int)(scan_word >> 32);
-        if ((unsigned)scan_word < level[ep & 1].nchunks) {
+        if (fmmgb::claimed_chunk(scan_word, level[ep & 1].chunks) >= 0) {
             x.st = CLAIM;
             return true;
         }
         if (pending < nw && try_raise())
             return true;
-        if (pending == 0 && scan_done >= (int)level[ep & 1].nchunks && w_tail == w_head && raise_lock == ep) {
+        if (pending == 0 && scan_done >= (int)(unsigned)level[ep & 1].chunks && w_tail == w_head && raise_lock == ep) {
             x.st = STOP;
             return true;
         }
@@ -172,13 +174,16 @@ struct Model {
         case CLAIM:
             x.claim = scan_word++;
             x.st = ACCEPT;
+            if (rnd(8) == 0)
+                x.away = rnd(40 * n);
             return true;
         case ACCEPT: {
             x.ep = (int)(x.claim >> 32);
             x.st = POLL;
-            if ((unsigned)x.claim < level[x.ep & 1].nchunks) {
-                x.ch = (int)(unsigned)x.claim;
-                if (seen[(size_t)x.ch]++)
+            const u64 chunks = level[x.ep & 1].chunks;
+            x.ch = fmmgb::claimed_chunk(any_raise ? ((chunks >> 32) << 32) | (unsigned)x.claim : x.claim, chunks);
+            if (x.ch >= 0) {
+                if ((u64)x.ch >= seen.size() || seen[(size_t)x.ch]++)
                     bad = "a chunk was taken twice";
                 x.i = 0;
                 x.kept = kNone;
@@ -331,7 +336,7 @@ struct Model {
 
 int main(int argc, char **argv)
 {
-    if (argc != 8)
+    if (argc != 9)
         return 1;
     const int n = atoi(argv[1]), waiting = atoi(argv[2]), warps = atoi(argv[3]), levels = atoi(argv[4]),
               release = atoi(argv[5]), seeds = atoi(argv[6]);
@@ -343,6 +348,7 @@ int main(int argc, char **argv)
         m.nw = warps;
         m.cap_q = (unsigned long long)n;
         m.cap_w = slots ? slots : fmmgb::waiting_slots(n);
+        m.any_raise = atoi(argv[8]) != 0;
         m.stride = release;
         m.budget = 4 * n;
         m.rng.seed((unsigned long long)s + 1);

@@ -1,6 +1,7 @@
 """The protocol of the one-launch brick scheduler as a host model
 (tests/host/scheduler_model.cpp: warps take turns at random, one atomic
-operation a turn) with the ring sizes of csrc/fmm_ring.h: it must always end."""
+operation a turn) with the ring sizes and the claims of csrc/fmm_ring.h: it must always
+end, with every chunk of a scan taken once."""
 import os
 import subprocess
 
@@ -17,8 +18,8 @@ def model(tmp_path_factory):
                     os.path.join(ROOT, "paper_1502_07303_gb300", "csrc"),
                     os.path.join(ROOT, "tests", "host", "scheduler_model.cpp"), "-o", exe], check=True)
 
-    def run(bricks, waiting, warps, levels=40, release=1, slots=0):
-        args = (bricks, waiting, warps, levels, release, SEEDS, slots)
+    def run(bricks, waiting, warps, levels=40, release=1, slots=0, any_raise=0):
+        args = (bricks, waiting, warps, levels, release, SEEDS, slots, any_raise)
         r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=300)
         return r.returncode, r.stdout
     return run
@@ -40,3 +41,16 @@ def test_one_slot_per_brick_would_stall(model):
     """The model does find a ring that is too small."""
     rc, out = model(512, 512, 4, slots=512)
     assert rc == 2, out
+
+
+# (few bricks wait at first: scans of one to a few chunks, and more of them later)
+@pytest.mark.parametrize("bricks,waiting,warps", [(300, 20, 16), (1000, 20, 32), (4000, 40, 64)])
+def test_late_claims_take_no_chunk(model, bricks, waiting, warps):
+    rc, out = model(bricks, waiting, warps)
+    assert rc == 0, out
+
+
+def test_claims_of_any_raise_would_take_chunks_twice(model):
+    """The model does find a claim that is taken for a later scan's."""
+    rc, out = model(1000, 20, 32, any_raise=1)
+    assert rc == 3 and "twice" in out, out
