@@ -450,9 +450,13 @@ __device__ __forceinline__ unsigned long long vloadu(const unsigned long long *p
 
 // Put brick b at position t of the ready queue or the waiting ring (waits,
 // bounded, for a queue slot still being read; the waiting ring has a free slot
-// for every append, fmm_ring.h).
+// for every append, fmm_ring.h).  own: a queue ticket this warp holds while it
+// scans, or -1.  Its entry would stay unread for as long as this waits, and the
+// slot waited for can be that very one (a raise that queues nearly every brick,
+// and marches that queue some again meanwhile): the wait takes the entry out,
+// into held.
 __device__ __forceinline__ void ring_put(Control *c, unsigned long long *q, unsigned long long cap,
-                                         unsigned long long t, long long b)
+                                         unsigned long long t, long long b, long long own, long long &held)
 {
     const unsigned long long v = ((t & 0xffffffffull) << 32) | (unsigned long long)(b + 1);
     unsigned long long *slot = q + (t % cap);
@@ -460,6 +464,12 @@ __device__ __forceinline__ void ring_put(Control *c, unsigned long long *q, unsi
         return;
     const unsigned long long ts = device_ns(), lim = vload(&c->wait_ns);
     while (atomicCAS(slot, 0ull, v) != 0ull) {
+        if (own >= 0) {
+            unsigned long long *mine = q + (unsigned long long)own % cap;
+            const unsigned long long e = vloadu(mine);
+            if (e != 0ull && (e >> 32) == ((unsigned long long)own & 0xffffffffull) && atomicCAS(mine, e, 0ull) == e)
+                held = (long long)(e & 0xffffffffull) - 1;
+        }
         if (device_ns() - ts > lim || (vload((const int *)&c->error) & ERR_SPIN)) {
             atomicOr(&c->error, ERR_SPIN);
             break;
@@ -593,10 +603,11 @@ __device__ __forceinline__ void finish_brick(const DeviceState &s, unsigned long
         tq = __shfl_sync(FULL, tq, 0);
         tw = __shfl_sync(FULL, tw, 0);
         const unsigned below = (1u << lane) - 1u;
+        long long none = -1;   // (a warp that marches holds no ticket)
         if (act == 1)
-            ring_put(c, s.queue, cap, tq + __popc(bq & below), tb);
+            ring_put(c, s.queue, cap, tq + __popc(bq & below), tb, -1, none);
         else if (act == 2)
-            ring_put(c, s.waiting, waiting_slots((long long)cap), tw + __popc(bw & below), tb);
+            ring_put(c, s.waiting, waiting_slots((long long)cap), tw + __popc(bw & below), tb, -1, none);
     }
     __syncwarp();
 }
@@ -844,9 +855,13 @@ __device__ void next_job(Control *c, unsigned long long *q, unsigned long long c
     job = 2;
 }
 
-// One warp scans a chunk of the waiting ring for the bound of raise ep.
-__device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long long cap, int ch, int ep, int lane)
+// One warp scans a chunk of the waiting ring for the bound of raise ep.  ticket:
+// the queue ticket the warp holds (or -1); returns the brick of that ticket if a
+// wait had to take it from the queue, else -1.
+__device__ __forceinline__ long long scan_chunk(const DeviceState &s, unsigned long long cap, int ch, int ep,
+                                                long long ticket, int lane)
 {
+    long long held = -1;
     Control *c = s.ctrl;
     const auto &lv = c->level[ep & 1];
     const unsigned long long end = vloadu(&lv.end), wcap = waiting_slots((long long)cap);
@@ -913,10 +928,11 @@ __device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long l
         tq = __shfl_sync(FULL, tq, 0);
         tw = __shfl_sync(FULL, tw, 0);
         const unsigned below = (1u << lane) - 1u;
+        long long none = -1;
         if (act == 1)
-            ring_put(c, s.queue, cap, tq + __popc(bq & below), b);
+            ring_put(c, s.queue, cap, tq + __popc(bq & below), b, ticket, held);
         else if (act == 2)
-            ring_put(c, s.waiting, wcap, tw + __popc(bw & below), b);
+            ring_put(c, s.waiting, wcap, tw + __popc(bw & below), b, -1, none);
     }
     kept = __reduce_min_sync(FULL, kept);
     if (lane == 0) {
@@ -925,7 +941,7 @@ __device__ __forceinline__ void scan_chunk(const DeviceState &s, unsigned long l
         __threadfence();
         atomicAdd(&c->scan_done, 1);
     }
-    __syncwarp();
+    return (long long)__reduce_max_sync(FULL, (unsigned)(held + 1)) - 1;   // a brick index has 31 bits
 }
 
 template <typename real, bool kHetero, bool kTape, bool kAniso, bool kBounded, bool kAll>
@@ -956,8 +972,10 @@ __global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape
             break;
         if (job == 1) {
             ep = __shfl_sync(FULL, ep, 0);
-            scan_chunk(s, cap, (int)arg, ep, lane);
-            continue;
+            arg = scan_chunk(s, cap, (int)arg, ep, __shfl_sync(FULL, ticket, 0), lane);
+            if (arg < 0)
+                continue;
+            ticket = -1;
         }
         const long long b = arg;
         long long nbi[kFaces];

@@ -6,11 +6,12 @@
 // launch is done (exit 0), when no warp can move (stalled, exit 2), or when a
 // chunk of a scan is taken twice, an entry is lost or work is left (exit 3).
 //
-//   scheduler_model bricks waiting warps levels release seeds ring_slots any_raise
+//   scheduler_model bricks waiting warps levels release seeds ring_slots any_raise keep
 //
 // waiting: bricks that wait at the start, their work spread over `levels`
 // strides; release: strides a raise goes up; ring_slots: slots of the waiting
-// ring (0: the library's); any_raise: 1 takes a claim without a look at its raise.
+// ring (0: the library's); any_raise: 1 takes a claim without a look at its raise;
+// keep: 1 leaves the entry of a scanning warp's own ticket where it is.
 #include "fmm_ring.h"
 
 #include <algorithm>
@@ -47,7 +48,7 @@ struct Warp {
     std::vector<int> act;
     std::vector<Put> puts;
     size_t at = 0;
-    int brick = -1;
+    int brick = -1, held = -1;
     std::vector<std::pair<int, int>> flags;    // brick, work
     long away = 0;
 };
@@ -56,7 +57,7 @@ struct Model {
     int n, nw;
     u64 cap_w, cap_q;
     int stride, budget;
-    bool any_raise = false;
+    bool any_raise = false, keep = false;
     std::mt19937_64 rng;
     std::vector<int> key, fl;
     std::vector<u64> queue, ring;
@@ -90,6 +91,16 @@ struct Model {
             const size_t j = (o + k) % x.puts.size();
             if (try_put(x.puts[j])) {
                 x.puts.erase(x.puts.begin() + (long)j);
+                return true;
+            }
+        }
+        // a scanning warp that waits for a queue slot takes its own ticket's
+        // entry out
+        if (!keep && x.ticket >= 0 && x.held < 0) {
+            u64 &s = queue[(u64)x.ticket % cap_q];
+            if (s && (s >> 32) == ((u64)x.ticket & 0xffffffffull)) {
+                x.held = (int)(s & 0xffffffffull) - 1;
+                s = 0;
                 return true;
             }
         }
@@ -235,6 +246,12 @@ struct Model {
             scan_min = std::min(scan_min, x.kept);
             ++scan_done;
             x.st = POLL;
+            if (x.held >= 0) {
+                x.brick = x.held;
+                x.held = -1;
+                x.ticket = -1;
+                x.st = TAKE;
+            }
             return true;
         case TAKE:
             key[(size_t)x.brick] = kNone;
@@ -336,7 +353,7 @@ struct Model {
 
 int main(int argc, char **argv)
 {
-    if (argc != 9)
+    if (argc != 10)
         return 1;
     const int n = atoi(argv[1]), waiting = atoi(argv[2]), warps = atoi(argv[3]), levels = atoi(argv[4]),
               release = atoi(argv[5]), seeds = atoi(argv[6]);
@@ -349,6 +366,7 @@ int main(int argc, char **argv)
         m.cap_q = (unsigned long long)n;
         m.cap_w = slots ? slots : fmmgb::waiting_slots(n);
         m.any_raise = atoi(argv[8]) != 0;
+        m.keep = atoi(argv[9]) != 0;
         m.stride = release;
         m.budget = 4 * n;
         m.rng.seed((unsigned long long)s + 1);

@@ -18,8 +18,8 @@ def model(tmp_path_factory):
                     os.path.join(ROOT, "paper_1502_07303_gb300", "csrc"),
                     os.path.join(ROOT, "tests", "host", "scheduler_model.cpp"), "-o", exe], check=True)
 
-    def run(bricks, waiting, warps, levels=40, release=1, slots=0, any_raise=0):
-        args = (bricks, waiting, warps, levels, release, SEEDS, slots, any_raise)
+    def run(bricks, waiting, warps, levels=40, release=1, slots=0, any_raise=0, keep=0):
+        args = (bricks, waiting, warps, levels, release, SEEDS, slots, any_raise, keep)
         r = subprocess.run([exe, *map(str, args)], capture_output=True, text=True, timeout=300)
         return r.returncode, r.stdout
     return run
@@ -54,3 +54,17 @@ def test_claims_of_any_raise_would_take_chunks_twice(model):
     """The model does find a claim that is taken for a later scan's."""
     rc, out = model(1000, 20, 32, any_raise=1)
     assert rc == 3 and "twice" in out, out
+
+
+@pytest.mark.parametrize("bricks,waiting,warps", GRIDS)
+@pytest.mark.parametrize("levels,release", [(1, 100), (3, 2)])
+def test_raises_that_queue_every_brick(model, bricks, waiting, warps, levels, release):
+    """Scanning warps hold queue tickets while the queue fills."""
+    rc, out = model(bricks, waiting, warps, levels=levels, release=release)
+    assert rc == 0, out
+
+
+def test_a_kept_ticket_entry_would_stall(model):
+    """The model does find a warp that waits for a slot only it can empty."""
+    rc, out = model(512, 512, 4, levels=1, release=100, keep=1)
+    assert rc == 2, out
