@@ -505,8 +505,10 @@ __device__ __forceinline__ unsigned work_key(float v) { return __float_as_uint(v
 __device__ __forceinline__ unsigned work_key(double v) { return __float_as_uint(__double2float_rd(v)); }
 
 // Take brick b from the queue: forget the work recorded so far, then read its
-// halo (acquire: the cells behind the recorded values are visible).  Returns
-// the changed faces (bit f), all ones for kWorkFull.
+// halo.  Lane 0 acquires, the barrier and the fence after it order every lane's
+// loads behind that (a shuffle alone orders no memory): the word is cleared, so a
+// load that missed a recorded value would lose it.  Returns the changed faces
+// (bit f), all ones for kWorkFull.
 __device__ __forceinline__ unsigned take_brick(const DeviceState &s, long long b, int lane)
 {
     unsigned fl = 0;
@@ -525,6 +527,8 @@ __device__ __forceinline__ unsigned take_brick(const DeviceState &s, long long b
         }
         fl = (unsigned)old;
     }
+    __syncwarp();
+    fence_acq_rel();
     fl = __shfl_sync(FULL, fl, 0);
     return (fl & kWorkFull) ? ~0u : fl / kWorkFace;
 }
@@ -862,6 +866,7 @@ __device__ __forceinline__ long long scan_chunk(const DeviceState &s, unsigned l
                                                 long long ticket, int lane)
 {
     long long held = -1;
+    __syncwarp();   // every lane's loads of the level come after lane 0's claim
     Control *c = s.ctrl;
     const auto &lv = c->level[ep & 1];
     const unsigned long long end = vloadu(&lv.end), wcap = waiting_slots((long long)cap);
