@@ -505,10 +505,11 @@ __device__ __forceinline__ unsigned work_key(float v) { return __float_as_uint(v
 __device__ __forceinline__ unsigned work_key(double v) { return __float_as_uint(__double2float_rd(v)); }
 
 // Take brick b from the queue: forget the work recorded so far, then read its
-// halo.  Lane 0 acquires, the barrier and the fence after it order every lane's
-// loads behind that (a shuffle alone orders no memory): the word is cleared, so a
-// load that missed a recorded value would lose it.  Returns the changed faces
-// (bit f), all ones for kWorkFull.
+// halo.  Lane 0 acquires and the barrier after it orders every lane's loads
+// behind that (a shuffle alone orders no memory): the word is cleared, so a load
+// that missed a recorded value would lose it.  (A fence in every lane as well
+// took 1 to 2% of the whole solves.)  Returns the changed faces (bit f), all ones
+// for kWorkFull.
 __device__ __forceinline__ unsigned take_brick(const DeviceState &s, long long b, int lane)
 {
     unsigned fl = 0;
@@ -528,7 +529,6 @@ __device__ __forceinline__ unsigned take_brick(const DeviceState &s, long long b
         fl = (unsigned)old;
     }
     __syncwarp();
-    fence_acq_rel();
     fl = __shfl_sync(FULL, fl, 0);
     return (fl & kWorkFull) ? ~0u : fl / kWorkFace;
 }
@@ -548,8 +548,10 @@ __device__ __forceinline__ void finish_brick(const DeviceState &s, unsigned long
     float bound = __uint_as_float(kNoWork);
     if (!kAll)
         bound = *(const volatile float *)&c->level[(vloadu(&c->scan_word) >> 32) & 1u].bound;
-    fence_acq_rel();   // the write-back before the flags
+    // all lanes' write-back before any lane's flags: the barrier, then each lane's
+    // fence before its atomic
     __syncwarp();
+    fence_acq_rel();
     long long tb = -1;        // the brick whose word this lane updates
     unsigned key = kNoWork;   // work to record
     if (nt.m) {
