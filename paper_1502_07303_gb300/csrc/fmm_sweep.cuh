@@ -574,15 +574,21 @@ __device__ __forceinline__ void sweep_brick(const Geom &g, const DeviceState &s,
     }
     __syncwarp();
     if (kBounded) {
-        // mark the cells no neighbour may use
+        // mark the cells no neighbour may use; a KNOWN cell among them (a solve
+        // stopped with bricks marched far beyond its bound and resumed with a
+        // lower one) is BAND again, so the brick is not KNOWN any more
+        bool marked = false;
 #pragma unroll 4
         for (int k = 0; k < 16; ++k) {
             const int c = lane + 32 * k, ti = mt_of(c);
             const uint8_t t = W.tg[c];
             const real v = W.kv[ti];
-            if ((t & ST_MASK) != ST_FIX && lt((t & TG_NEG) ? bound0 : bound1, v))
+            if ((t & ST_MASK) != ST_FIX && lt((t & TG_NEG) ? bound0 : bound1, v)) {
                 W.kv[ti] = kmark(v);
+                marked = true;
+            }
         }
+        was_known = !__any_sync(FULL, marked) && was_known;
         __syncwarp();
     }
 
