@@ -1010,11 +1010,12 @@ __global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape
 }
 
 // Seed a launch: the work word of every brick from its BAND minima and the
-// work a stopped launch left, queued (at or below the bound) or waiting.
+// work a stopped launch left, queued (at or below the bound) or waiting.  A brick
+// that a stopped phased solve left dirty is queued (the value is not recorded).
 // all: the bound of each side is fixed and nothing waits.
 template <typename real>
 __global__ void k_seed(Geom g, const real *__restrict__ bmin, Control *ctrl, unsigned long long *work,
-                       unsigned long long *q, unsigned long long *waiting, double width, bool all)
+                       unsigned *dirty, unsigned long long *q, unsigned long long *waiting, double width, bool all)
 {
     if (ctrl->done)
         return;
@@ -1051,6 +1052,10 @@ __global__ void k_seed(Geom g, const real *__restrict__ bmin, Control *ctrl, uns
                     key = umin(key, work_key(m));
                 if (key < kNoWork)
                     act = __uint_as_float(key) <= bd ? 1 : 2;
+            }
+            if (dirty[b] != 0u) {
+                dirty[b] = 0u;
+                act = 1;
             }
             work[b] = work_word(key, kWorkFull | (act == 1 ? kWorkActive : (act == 2 ? kWorkWaiting : 0u)));
         }
@@ -1165,11 +1170,12 @@ __global__ void k_control(Control *c, double width, double stride, long long max
 }
 
 // Work lists: list 0 = bricks with a BAND cell at or below the bound or with
-// pending overlap changes (first march); list 1 = bricks with pending changes
+// pending overlap changes (first march), those a stopped one-launch solve left in
+// the work words among them; list 1 = bricks with pending changes
 // (second march, after the exchange).  Changes flagged during the march are
 // left for the next selection.
 template <typename real>
-__global__ void k_select(Geom g, const real *__restrict__ bmin, unsigned *dirty,
+__global__ void k_select(Geom g, const real *__restrict__ bmin, unsigned *dirty, unsigned long long *work,
                          Control *ctrl, int *list, int which)
 {
     if (ctrl->done)
@@ -1189,6 +1195,10 @@ __global__ void k_select(Geom g, const real *__restrict__ bmin, unsigned *dirty,
                 // of bricks without BAND cells)
                 const double m0 = (double)bmin[2 * b], m1 = (double)bmin[2 * b + 1];
                 sel = sel || (m0 < CUDART_INF && m0 <= bd0) || (m1 < CUDART_INF && m1 <= bd1);
+                if ((unsigned)(work[b] >> 32) < kNoWork) {
+                    sel = true;
+                    work[b] = ~0ull;
+                }
             }
         }
         if (dty)
@@ -1611,7 +1621,7 @@ cudaError_t restart_impl(const Geom &g, const DeviceState &s, const SolveParams 
     k_control<<<1, 1, 0, st>>>(s.ctrl, p.width, p.stride, p.max_restarts);
     if (one_launch_schedule(p.schedule)) {
         const bool all = p.schedule == kSchedulePersistent;
-        k_seed<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.ctrl, s.work, s.queue, s.waiting, p.width, all);
+        k_seed<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.ctrl, s.work, s.dirty, s.queue, s.waiting, p.width, all);
         if (trace)
             k_trace_seed<<<1, 1, 0, st>>>(s.ctrl, trace);
         if (ev)
@@ -1625,7 +1635,7 @@ cudaError_t restart_impl(const Geom &g, const DeviceState &s, const SolveParams 
         const int which = pass == 0 ? 0 : 1;
         if (pass >= 2)
             k_reset_list<<<1, 1, 0, st>>>(s.ctrl, 1);
-        k_select<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.dirty, s.ctrl, s.list[which], which);
+        k_select<real><<<rb, 256, 0, st>>>(g, (const real *)s.bmin, s.dirty, s.work, s.ctrl, s.list[which], which);
         if (trace)
             k_trace<<<1, 1, 0, st>>>(s.ctrl, which, pass, trace + 3 * pass);
         if (ev)
@@ -1809,11 +1819,11 @@ cudaError_t launch_march_to(int dtype, const Geom &g, const DeviceState &s, cons
     k_set_bound<<<1, 1, 0, st>>>(s.ctrl, b0, b1);
     const int rb = grid_for(g.nbricks, 256, 4096);
     if (dtype == 1) {
-        k_seed<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.ctrl, s.work, s.queue, s.waiting, p.width,
+        k_seed<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.ctrl, s.work, s.dirty, s.queue, s.waiting, p.width,
                                            true);
         queue_march<double>(g, s, p, true, st);
     } else {
-        k_seed<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.ctrl, s.work, s.queue, s.waiting, p.width, true);
+        k_seed<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.ctrl, s.work, s.dirty, s.queue, s.waiting, p.width, true);
         queue_march<float>(g, s, p, true, st);
     }
     return cudaGetLastError();
@@ -1837,9 +1847,9 @@ cudaError_t launch_select(int dtype, const Geom &g, const DeviceState &s, int wh
 {
     const int rb = grid_for(g.nbricks, 256, 4096);
     if (dtype == 1)
-        k_select<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.dirty, s.ctrl, s.list[which], which);
+        k_select<double><<<rb, 256, 0, st>>>(g, (const double *)s.bmin, s.dirty, s.work, s.ctrl, s.list[which], which);
     else
-        k_select<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.dirty, s.ctrl, s.list[which], which);
+        k_select<float><<<rb, 256, 0, st>>>(g, (const float *)s.bmin, s.dirty, s.work, s.ctrl, s.list[which], which);
     return cudaGetLastError();
 }
 
