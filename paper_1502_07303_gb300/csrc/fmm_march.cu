@@ -234,24 +234,42 @@ __device__ __forceinline__ unsigned every_fourth(unsigned v)
     return (v | (v >> 12)) & 0xffu;
 }
 
-// Algorithm 8 for brick (bx, by, bz) of a level set, by one warp.  Almost no
-// cell is at the interface, and telling which takes only signs: a lane reads
-// the 16 cells of its slots (x = lane & 7, y = lane / 8 + 4 (k & 1), z = k / 2)
-// and 12 cells of the face halo, keeps their signs as bits, and gets the
-// neighbours' signs by shifts, shuffles and ballots; reinit_load / reinit_eval
-// run for the interface cells alone.  28 loads a lane instead of 112, and a
-// tenth of the instructions.  Against seven loads for every cell, whole
-// solves: 1024^3 in double 58.5 -> 56.1 ms (that pass took 7.3 ms; HBM alone
-// 2.7), 256 grids of 32^3 to 192^3 in float 16.3 -> 15.0 ms (2.2; HBM 0.5).
+// Algorithm 8 takes two phases over the bricks of a CTA.  Almost no cell is at
+// the interface, and telling which takes only signs: in the first phase one warp
+// per brick has a lane read the 16 cells of its slots (x = lane & 7, y = lane / 8 +
+// 4 (k & 1), z = k / 2) and 12 cells of the face halo, keep their signs as bits,
+// and get the neighbours' signs by shifts, shuffles and ballots; the other cells
+// are written at once.  The interface cells of all bricks of the CTA go to one
+// list, and in the second phase the CTA's threads run reinit_load / reinit_eval on
+// it: a cell takes a chain of IEEE divisions and a root (5 us in double), so a
+// brick's 100 to 200 of them are spread over the CTA.
+// This kernel, float / double: 33x36x40 (150 bricks, one per CTA) 6.0 / 13.3 us,
+// 256^3 48 / 118 us.  With one cell a thread and seven loads for each 5.0 / 17.5 and
+// 103 / 298 us; with each lane of the first phase evaluating its own interface
+// cells 14.3 / 52.6 and 56 / 194 us.  Whole solves against that last form:
+// 1024^3 in double 56.5 -> 55.3 ms, 256 grids of 32^3 to 192^3 in float the same.
+// One brick of a level set: the caller's array with its sizes and cell sizes (a
+// subdomain's layers beyond its own, see above) and the brick's coordinates.
 template <typename real>
-__device__ __forceinline__ void reinit_brick(const real *__restrict__ phi, int nx, int ny, int nz, int bx,
-                                             int by, int bz, double hx, double hy, double hz, int zlo,
-                                             int zhi, real *__restrict__ T, uint8_t *__restrict__ tag)
+struct ReinitBrick {
+    const real *phi;
+    int nx, ny, nz, bx, by, bz;
+    double hx, hy, hz;
+    int zlo, zhi;
+};
+
+// First phase, one warp: writes the cells that are not at the interface, returns
+// the slots of this lane that are.
+template <typename real>
+__device__ __forceinline__ unsigned reinit_signs(const ReinitBrick<real> &B, real *__restrict__ T,
+                                                 uint8_t *__restrict__ tag)
 {
+    const real *__restrict__ phi = B.phi;
+    const int nx = B.nx, ny = B.ny, nz = B.nz, bx = B.bx, by = B.by, zlo = B.zlo, zhi = B.zhi;
     constexpr unsigned kAll = 0xffffffffu, kEven = 0x5555u, kOdd = 0xaaaau;
     const int lane = threadIdx.x & 31, lx = lane & 7, lr = lane >> 3;
     const long long sy = nx, sz = (long long)nx * ny;
-    const int i0 = bx * kB, j0 = by * kB, k0 = bz * kB;
+    const int i0 = bx * kB, j0 = by * kB, k0 = B.bz * kB;
     const int i = i0 + lx, j = j0 + lr;
     const real *col = phi + (long long)k0 * sz + (long long)j * sy + i;
     const bool in_x = i < nx, in_y0 = in_x && j < ny, in_y1 = in_x && j + 4 < ny;
@@ -320,29 +338,71 @@ __device__ __forceinline__ void reinit_brick(const real *__restrict__ phi, int n
                              : ((S >> k) & 1u) ? (uint8_t)ST_FAR
                                                : (uint8_t)(ST_FAR | TG_NEG);
     }
-    for (unsigned m = cross; m; m &= m - 1u) {
-        const int k = __ffs(m) - 1;
+    return cross;
+}
+
+// Both phases for bricks first .. first + count - 1 (at most one per warp of the
+// CTA): info(b) gives a brick, or a null phi for one without a level set, whose
+// cells it has written.
+struct ReinitList {
+    int n;
+    uint16_t cell[kInitThreads / 32 * kB3];   // warp of the brick << 9 | cell
+};
+template <typename real, typename Info>
+__device__ __forceinline__ void reinit_bricks(int first, int count, Info &&info, real *__restrict__ T,
+                                              uint8_t *__restrict__ tag, ReinitList &L)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (threadIdx.x == 0)
+        L.n = 0;
+    __syncthreads();
+    if (warp < count) {
+        const ReinitBrick<real> B = info(first + warp);
+        const long long base = (long long)(first + warp) * kB3;
+        const unsigned cross = B.phi ? reinit_signs<real>(B, T + base, tag + base) : 0u;
+        const int cnt = __popc(cross);
+        int pre = cnt;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(0xffffffffu, pre, o);
+            if (lane >= o)
+                pre += t;
+        }
+        int at = 0;
+        if (lane == 31 && pre)
+            at = atomicAdd(&L.n, pre);
+        at = __shfl_sync(0xffffffffu, at, 31) + pre - cnt;
+        for (unsigned m = cross; m; m &= m - 1u)
+            L.cell[at++] = (uint16_t)(warp << 9 | (lane + 32 * (__ffs(m) - 1)));
+    }
+    __syncthreads();
+    for (int l = threadIdx.x; l < L.n; l += blockDim.x) {
+        const int b = first + (L.cell[l] >> 9), c = L.cell[l] & (kB3 - 1);
+        const ReinitBrick<real> B = info(b);
         real fc, fn[6], Tv;
         uint8_t tg;
-        reinit_load<real>(phi, nx, ny, nz, i, j + 4 * (k & 1), k0 + (k >> 1), zlo, zhi, fc, fn);
-        reinit_eval<real>(fc, fn, hx, hy, hz, Tv, tg);
-        T[lane + 32 * k] = Tv;
-        tag[lane + 32 * k] = tg;
+        reinit_load<real>(B.phi, B.nx, B.ny, B.nz, B.bx * kB + (c & 7), B.by * kB + ((c >> 3) & 7),
+                          B.bz * kB + (c >> 6), B.zlo, B.zhi, fc, fn);
+        reinit_eval<real>(fc, fn, B.hx, B.hy, B.hz, Tv, tg);
+        T[(long long)b * kB3 + c] = Tv;
+        tag[(long long)b * kB3 + c] = tg;
     }
+    __syncthreads();   // the list of the next bricks
 }
 
 template <typename real>
 __global__ void __launch_bounds__(kInitThreads) k_init_reinit(Geom g, double hx, double hy, double hz,
                                                               const real *__restrict__ phi, real *T,
-                                                              uint8_t *tag, int zlo, int zhi)
+                                                              uint8_t *tag, int zlo, int zhi, int group)
 {
-    const int warps = gridDim.x * (kInitThreads / 32);
-    for (int b = blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5); b < (int)g.nbricks; b += warps) {
-        int bx, by, bz;
-        brick_xyz32(g, b, bx, by, bz);
-        reinit_brick<real>(phi, g.nx, g.ny, g.nz, bx, by, bz, hx, hy, hz, zlo, zhi, T + (long long)b * kB3,
-                           tag + (long long)b * kB3);
-    }
+    __shared__ ReinitList list;
+    const auto info = [&](int b) {
+        ReinitBrick<real> B = {phi, g.nx, g.ny, g.nz, 0, 0, 0, hx, hy, hz, zlo, zhi};
+        brick_xyz32(g, b, B.bx, B.by, B.bz);
+        return B;
+    };
+    for (long long b = (long long)blockIdx.x * group; b < g.nbricks; b += (long long)gridDim.x * group)
+        reinit_bricks<real>((int)b, (int)min((long long)group, g.nbricks - b), info, T, tag, list);
 }
 
 // Speed field to brick layout: the speed term (h/F)^2 of the shifted solve
@@ -1374,32 +1434,33 @@ __device__ __forceinline__ void batch_cell(const BatchGrid &G, long long b, int 
     k = bz * kB + (c >> 6);
 }
 
-// Algorithm 8 for every grid of a batch, one warp per brick: a grid with a
-// level set gets its interface cells (reinit_brick), a grid of point sources
-// starts all FAR (k_batch_sources then fixes its sources).
+// Algorithm 8 for every grid of a batch: a grid with a level set gets its
+// interface cells, a grid of point sources starts all FAR (k_batch_sources then
+// fixes its sources).
 template <typename real>
 __global__ void __launch_bounds__(kInitThreads) k_batch_init(const BatchGrid *__restrict__ grids,
                                                              const int *__restrict__ bgrid, int nbricks,
-                                                             real *__restrict__ T, uint8_t *__restrict__ tag)
+                                                             real *__restrict__ T, uint8_t *__restrict__ tag,
+                                                             int group)
 {
-    const int warps = gridDim.x * (kInitThreads / 32), lane = threadIdx.x & 31;
-    for (int b = blockIdx.x * (kInitThreads / 32) + (threadIdx.x >> 5); b < nbricks; b += warps) {
+    __shared__ ReinitList list;
+    const auto info = [&](int b) {
         const BatchGrid &G = grids[bgrid[b]];
-        const long long base = (long long)b * kB3;
+        int i, j, k;
         if (G.phi0) {
-            int i, j, k;
             batch_cell(G, b, 0, i, j, k);
-            reinit_brick<real>((const real *)G.phi0, G.nx, G.ny, G.nz, i / kB, j / kB, k / kB, G.h, G.h, G.h, 0, 0,
-                               T + base, tag + base);
-            continue;
+            return ReinitBrick<real>{(const real *)G.phi0, G.nx, G.ny, G.nz, i / kB, j / kB, k / kB, G.h, G.h, G.h, 0, 0};
         }
-        for (int c = lane; c < kB3; c += 32) {
-            int i, j, k;
+        const long long base = (long long)b * kB3;
+        for (int c = threadIdx.x & 31; c < kB3; c += 32) {
             batch_cell(G, b, c, i, j, k);
             T[base + c] = inf_v<real>();
             tag[base + c] = i < G.nx && j < G.ny && k < G.nz ? ST_FAR : TG_OUT | ST_FAR;
         }
-    }
+        return ReinitBrick<real>{};
+    };
+    for (long long b = (long long)blockIdx.x * group; b < nbricks; b += (long long)gridDim.x * group)
+        reinit_bricks<real>((int)b, (int)min((long long)group, nbricks - b), info, T, tag, list);
 }
 
 // The point sources of the batch: psi = 0, FIX (Algorithm 8).
@@ -1499,6 +1560,14 @@ int grid_for(long long n, int threads, int cap)
     if (b > cap)
         b = cap;
     return (int)b;
+}
+
+// Bricks per CTA of Algorithm 8: one per warp, fewer where the bricks would
+// otherwise fill only some of the 152 SMs.
+int init_group(long long nbricks)
+{
+    const long long n = nbricks / 152;
+    return (int)(n < 1 ? 1 : (n > kInitThreads / 32 ? kInitThreads / 32 : n));
 }
 
 template <typename real, bool kTape>
@@ -1729,14 +1798,14 @@ cudaError_t launch_init_reinit(int dtype, const Geom &g, const DeviceState &s,
                                const SolveParams &p, const void *phi0, cudaStream_t st, int zlo,
                                int zhi)
 {
-    const int nb = grid_for(g.nbricks, kInitThreads / 32, 152 * 16);
+    const int gr = init_group(g.nbricks), nb = grid_for(g.nbricks, gr, 152 * 16);
     const long long layer = (long long)g.nx * g.ny;
     if (dtype == 1)
         k_init_reinit<double><<<nb, kInitThreads, 0, st>>>(g, p.h, p.hy, p.hz, (const double *)phi0 + zlo * layer,
-                                                  (double *)s.T, s.tag, zlo, zhi);
+                                                  (double *)s.T, s.tag, zlo, zhi, gr);
     else
         k_init_reinit<float><<<nb, kInitThreads, 0, st>>>(g, p.h, p.hy, p.hz, (const float *)phi0 + zlo * layer,
-                                                 (float *)s.T, s.tag, zlo, zhi);
+                                                 (float *)s.T, s.tag, zlo, zhi, gr);
     return cudaGetLastError();
 }
 
@@ -1862,11 +1931,11 @@ cudaError_t launch_reset_list(const DeviceState &s, int which, cudaStream_t st)
 cudaError_t launch_batch_init(int dtype, const BatchGrid *grids, const int *bgrid,
                               long long nbricks, const DeviceState &s, cudaStream_t st)
 {
-    const int nb = grid_for(nbricks, kInitThreads / 32, 152 * 16);
+    const int gr = init_group(nbricks), nb = grid_for(nbricks, gr, 152 * 16);
     if (dtype == 1)
-        k_batch_init<double><<<nb, kInitThreads, 0, st>>>(grids, bgrid, (int)nbricks, (double *)s.T, s.tag);
+        k_batch_init<double><<<nb, kInitThreads, 0, st>>>(grids, bgrid, (int)nbricks, (double *)s.T, s.tag, gr);
     else
-        k_batch_init<float><<<nb, kInitThreads, 0, st>>>(grids, bgrid, (int)nbricks, (float *)s.T, s.tag);
+        k_batch_init<float><<<nb, kInitThreads, 0, st>>>(grids, bgrid, (int)nbricks, (float *)s.T, s.tag, gr);
     return cudaGetLastError();
 }
 
