@@ -472,7 +472,7 @@ fmm_status run_cell(fmm_handle *hd, void *T_out, uint8_t *tags_out)
     const auto t0 = std::chrono::steady_clock::now();
     const double limit_s = hd->cfg.timeout_s > 0 ? (double)hd->cfg.timeout_s : 600.0;
     bool timed_out = false, limited = false;
-    long long step = 0, batch = 1;
+    long long step = 0, batch = 16;   // (a small grid takes some 50 steps in all)
     for (;;) {
         long long n = batch;
         if (p.max_restarts > 0 && step + n > p.max_restarts)

@@ -368,18 +368,22 @@ __global__ void __launch_bounds__(kCellThreads) k_cell_apply(Geom g, real *T, ui
 // visits the bricks with a BAND cell at or below the step's limit and their
 // face neighbours (active bricks; CTA i owns the bricks i, i + CTAs, ..., so
 // neighbours lie on different SMs, its threads look at the BAND minima of
-// their bricks and the neighbours, and its warps share the active ones).
+// their bricks and the neighbours).
 //   relax : acceptance is evaluated, not stored (a BAND cell at or below its
-//           limit counts as KNOWN), and the cells next to an accepted one are
-//           packed 32 to a warp step and solved into `next`;
+//           limit counts as KNOWN).  A warp stages an active brick and lists the
+//           cells next to an accepted one; the cells of all its bricks are then
+//           tested and solved into `next` by the threads of the whole CTA (a
+//           step has one or two active bricks a CTA, and a warp with a brick of
+//           its own would test and solve its 100 cells in turn);
 //   apply : accepted cells become KNOWN, new values are applied, the brick's
 //           BAND minima and the global ones are renewed.
 // The solves read the same state as when every step streamed the whole grid in
-// three launches, so the results are the same bits.  128^3 in double, 4
-// spheres, 1094 steps: streaming took 93 ms (29 us a launch, bound by memory
-// latency at 1.3 TB/s and by the launches), this takes 35 ms: 32 us a step,
-// which is the slowest CTA's chain (stage, select, solve, two grid barriers);
-// the FP64 solves of the few bricks at the front fill a small part of it.
+// three launches, so the results are the same bits.  Spheres, second order, in
+// double: 128^3 (1230 steps) 98.8 ms streaming, 38.6 with a warp per brick to the
+// end of the phase, 32.9 so; 32^3 (180 steps) 4.6, 5.4, 3.9 ms.  A step is the
+// slowest CTA's chain (stage, list, solve, two grid barriers): 20 us on the
+// smallest grids, 27 on 128^3.  (On 32^3 in float, where a streamed step took
+// 18 us, it is 1.18 against 1.07 ms in first order, 59 steps.)
 // ---------------------------------------------------------------------------
 constexpr int kStepWarps = 16;
 
@@ -388,8 +392,14 @@ struct StepTile {
     real T[kTile3];          // brick and face halo
     uint8_t st[kTile3];      // 0 not usable, 1 KNOWN or FIX before the step, 3 accepted in it
     alignas(16) uint8_t tg[kB3];
-    uint16_t list[kB3];
     unsigned sel[32];        // per lane: cells next to an accepted halo cell
+};
+// What the warps of a CTA share in the relax phase: a brick's tile per warp, and
+// the cells of all of them (warp << 9 | cell) to test and to solve.
+template <typename real>
+struct StepSmem {
+    StepTile<real> tile[kStepWarps];
+    uint16_t test[kStepWarps * kB3], solve[kStepWarps * kB3];
 };
 
 __device__ __forceinline__ unsigned long long ldu(const unsigned long long *p)
@@ -505,7 +515,8 @@ __global__ void __launch_bounds__(kStepWarps * 32)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    StepTile<real> &W = reinterpret_cast<StepTile<real> *>(smem_raw)[warp];
+    StepSmem<real> &sm = *reinterpret_cast<StepSmem<real> *>(smem_raw);
+    StepTile<real> &W = sm.tile[warp];
     __shared__ unsigned long long bm[2];
     const real INF = inf_r<real>();
     const real wax[3] = {(real)1, (real)wy, (real)wz};
@@ -514,7 +525,7 @@ __global__ void __launch_bounds__(kStepWarps * 32)
     const long long owned = first < g.nbricks ? (g.nbricks - first + stride - 1) / stride : 0;
     constexpr int kThreadsStep = kStepWarps * 32;
     __shared__ unsigned alist[kThreadsStep];   // active bricks of a chunk
-    __shared__ int an;
+    __shared__ int an, n_test, n_solve;
     const float bucket_up = (float)bucket * 1.000001f;
     unsigned target = 0;
     unsigned long long accepted = 0, solves = 0;
@@ -564,100 +575,119 @@ __global__ void __launch_bounds__(kStepWarps * 32)
                     alist[atomicAdd(&an, 1)] = (unsigned)b;
             }
             __syncthreads();
-            for (int ai = warp; ai < an; ai += kStepWarps) {
-                const long long b = alist[ai], base = b * kB3;
-                int bx, by, bz;
-                brick_at(g, b, bx, by, bz);
-                const Limits<real> lb = brick_limits(bdelta[b], bucket, width, m, has);
-                // the brick and its halo, with what each cell is in this step
-                __syncwarp();
-                reinterpret_cast<uint4 *>(W.tg)[lane] = __ldcg(reinterpret_cast<const uint4 *>(tag + base) + lane);
-                W.sel[lane] = 0u;
-                real v[16];
+            for (int a0 = 0; a0 < an; a0 += kStepWarps) {
+                if (threadIdx.x == 0)
+                    n_test = n_solve = 0;
+                __syncthreads();
+                if (a0 + warp < an) {
+                    const long long b = alist[a0 + warp], base = b * kB3;
+                    int bx, by, bz;
+                    brick_at(g, b, bx, by, bz);
+                    const Limits<real> lb = brick_limits(bdelta[b], bucket, width, m, has);
+                    // the brick and its halo, with what each cell is in this step
+                    __syncwarp();
+                    reinterpret_cast<uint4 *>(W.tg)[lane] = __ldcg(reinterpret_cast<const uint4 *>(tag + base) + lane);
+                    W.sel[lane] = 0u;
+                    real v[16];
 #pragma unroll
-                for (int k = 0; k < 16; ++k)
-                    v[k] = __ldcg(T + base + lane + 32 * k);
-                __syncwarp();
-                unsigned acc = 0;
+                    for (int k = 0; k < 16; ++k)
+                        v[k] = __ldcg(T + base + lane + 32 * k);
+                    // (all loads first)
+                    real hv[12];
+                    uint8_t ht[12];
+                    real hd[6];
 #pragma unroll
-                for (int k = 0; k < 16; ++k) {
-                    const int c = lane + 32 * k, ti = tile_of(c);
-                    const int st = cell_state(W.tg[c], v[k], lb);
-                    W.T[ti] = v[k];
-                    W.st[ti] = (uint8_t)st;
-                    acc |= (unsigned)(st == 3) << k;
-                }
-                // (all loads first)
-                real hv[12];
-                uint8_t ht[12];
-                real hd[6];
+                    for (int f = 0; f < 6; ++f) {
+                        const long long nb = brick_next(g, bx, by, bz, f);
+                        hd[f] = nb >= 0 ? bdelta[nb] : (real)0;
 #pragma unroll
-                for (int f = 0; f < 6; ++f) {
-                    const long long nb = brick_next(g, bx, by, bz, f);
-                    hd[f] = nb >= 0 ? bdelta[nb] : (real)0;
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const long long e = nb * kB3 + face_cell(f ^ 1, lane + 32 * h);
-                        hv[2 * f + h] = nb >= 0 ? __ldcg(T + e) : INF;
-                        ht[2 * f + h] = nb >= 0 ? __ldcg(tag + e) : (uint8_t)(TG_OUT | ST_FAR);
-                    }
-                }
-#pragma unroll
-                for (int f = 0; f < 6; ++f) {
-                    const Limits<real> ln = brick_limits(hd[f], bucket, width, m, has);
-#pragma unroll
-                    for (int h = 0; h < 2; ++h) {
-                        const int st = cell_state(ht[2 * f + h], hv[2 * f + h], ln);
-                        const int hi = tile_of(face_cell(f, lane + 32 * h)) + ((f & 1) ? off[f >> 1] : -off[f >> 1]);
-                        W.T[hi] = hv[2 * f + h];
-                        W.st[hi] = (uint8_t)st;
-                        if (st == 3) {
-                            const int c = face_cell(f, lane + 32 * h);
-                            atomicOr(&W.sel[c & 31], 1u << (c >> 5));
+                        for (int h = 0; h < 2; ++h) {
+                            const long long e = nb * kB3 + face_cell(f ^ 1, lane + 32 * h);
+                            hv[2 * f + h] = nb >= 0 ? __ldcg(T + e) : INF;
+                            ht[2 * f + h] = nb >= 0 ? __ldcg(tag + e) : (uint8_t)(TG_OUT | ST_FAR);
                         }
                     }
+                    __syncwarp();
+                    unsigned acc = 0, open = 0;   // accepted in this step; not FIX or padding
+#pragma unroll
+                    for (int k = 0; k < 16; ++k) {
+                        const int c = lane + 32 * k, ti = tile_of(c);
+                        const uint8_t t = W.tg[c];
+                        const int st = cell_state(t, v[k], lb);
+                        open |= (unsigned)(!(t & TG_OUT) && (t & ST_MASK) != ST_FIX) << k;
+                        W.T[ti] = v[k];
+                        W.st[ti] = (uint8_t)st;
+                        acc |= (unsigned)(st == 3) << k;
+                    }
+#pragma unroll
+                    for (int f = 0; f < 6; ++f) {
+                        const Limits<real> ln = brick_limits(hd[f], bucket, width, m, has);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const int st = cell_state(ht[2 * f + h], hv[2 * f + h], ln);
+                            const int hi = tile_of(face_cell(f, lane + 32 * h)) + ((f & 1) ? off[f >> 1] : -off[f >> 1]);
+                            W.T[hi] = hv[2 * f + h];
+                            W.st[hi] = (uint8_t)st;
+                            if (st == 3) {
+                                const int c = face_cell(f, lane + 32 * h);
+                                atomicOr(&W.sel[c & 31], 1u << (c >> 5));
+                            }
+                        }
+                    }
+                    __syncwarp();
+                    // the cells next to an accepted one
+                    const unsigned cand = (neighbour_mask(acc, lane) | W.sel[lane]) & open;
+                    const int cnt = __popc(cand);
+                    int pre = cnt;
+#pragma unroll
+                    for (int o = 1; o < 32; o <<= 1) {
+                        const int t = __shfl_up_sync(FULL, pre, o);
+                        if (lane >= o)
+                            pre += t;
+                    }
+                    int at = 0;
+                    if (lane == 31 && pre)
+                        at = atomicAdd(&n_test, pre);
+                    at = __shfl_sync(FULL, at, 31) + pre - cnt;
+                    for (unsigned q = cand; q; q &= q - 1u)
+                        sm.test[at++] = (uint16_t)(warp << 9 | (lane + 32 * (__ffs((int)q) - 1)));
                 }
-                __syncwarp();
-                // the cells to solve: next to an accepted cell and above it
-                unsigned sel = 0;
-                for (unsigned q = neighbour_mask(acc, lane) | W.sel[lane]; q; q &= q - 1u) {
-                    const int k = __ffs((int)q) - 1, c = lane + 32 * k, ti = tile_of(c);
-                    const uint8_t t = W.tg[c];
-                    if ((t & TG_OUT) || (t & ST_MASK) == ST_FIX)
-                        continue;
-                    const real Tc = W.T[ti];
+                __syncthreads();
+                // of them, the cells above an accepted neighbour
+                for (int j0 = 32 * warp; j0 < n_test; j0 += kThreadsStep) {
+                    const int i = j0 + lane;
+                    const int e = i < n_test ? sm.test[i] : 0;
+                    const StepTile<real> &X = sm.tile[e >> 9];
+                    const int ti = tile_of(e & (kB3 - 1));
+                    const real Tc = X.T[ti];
                     bool trig = false;
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
-                        trig = trig || (W.st[ti - off[a]] == 3 && blt(W.T[ti - off[a]], Tc));
-                        trig = trig || (W.st[ti + off[a]] == 3 && blt(W.T[ti + off[a]], Tc));
+                        trig = trig || (X.st[ti - off[a]] == 3 && blt(X.T[ti - off[a]], Tc));
+                        trig = trig || (X.st[ti + off[a]] == 3 && blt(X.T[ti + off[a]], Tc));
                     }
-                    sel |= (unsigned)trig << k;
+                    const unsigned bal = __ballot_sync(FULL, trig && i < n_test);
+                    int at = 0;
+                    if (lane == 0 && bal)
+                        at = atomicAdd(&n_solve, __popc(bal));
+                    at = __shfl_sync(FULL, at, 0) + __popc(bal & ((1u << lane) - 1u));
+                    if (trig && i < n_test)
+                        sm.solve[at] = (uint16_t)e;
                 }
-                const int cnt = __popc(sel);
-                int pre = cnt;
-#pragma unroll
-                for (int o = 1; o < 32; o <<= 1) {
-                    const int t = __shfl_up_sync(FULL, pre, o);
-                    if (lane >= o)
-                        pre += t;
-                }
-                const int n = __shfl_sync(FULL, pre, 31);
-                pre -= cnt;
-                for (unsigned q = sel; q; q &= q - 1u)
-                    W.list[pre++] = (uint16_t)(lane + 32 * (__ffs((int)q) - 1));
-                __syncwarp();
-                solves += lane == 0 ? (unsigned)n : 0u;
-                for (int i = lane; i < n; i += 32) {
-                    const int c = W.list[i], ti = tile_of(c);
-                    const real Tc = W.T[ti];
+                __syncthreads();
+                solves += threadIdx.x == 0 ? (unsigned)n_solve : 0u;
+                for (int i = threadIdx.x; i < n_solve; i += kThreadsStep) {
+                    const int e = sm.solve[i], c = e & (kB3 - 1), ti = tile_of(c);
+                    const StepTile<real> &X = sm.tile[e >> 9];
+                    const long long b = alist[a0 + (e >> 9)], base = b * kB3;
+                    const real Tc = X.T[ti];
                     const int cc[3] = {c & 7, (c >> 3) & 7, c >> 6};
                     real psi[3] = {(real)0, (real)0, (real)0}, wt[3] = {(real)0, (real)0, (real)0};
                     unsigned axes = 0;
 #pragma unroll
                     for (int a = 0; a < 3; ++a) {
-                        const bool km = W.st[ti - off[a]] != 0, kp = W.st[ti + off[a]] != 0;
-                        const real vm = km ? W.T[ti - off[a]] : INF, vp = kp ? W.T[ti + off[a]] : INF;
+                        const bool km = X.st[ti - off[a]] != 0, kp = X.st[ti + off[a]] != 0;
+                        const real vm = km ? X.T[ti - off[a]] : INF, vp = kp ? X.T[ti + off[a]] : INF;
                         int d = 0;
                         if (km && blt(vm, Tc))
                             d = -1;
@@ -679,9 +709,11 @@ __global__ void __launch_bounds__(kStepWarps * 32)
                             real v2 = (real)0;
                             const int c2 = cc[a] + 2 * d;
                             if (c2 >= -1 && c2 <= kB) {
-                                k2 = W.st[ti + 2 * d * off[a]] != 0;
-                                v2 = W.T[ti + 2 * d * off[a]];
+                                k2 = X.st[ti + 2 * d * off[a]] != 0;
+                                v2 = X.T[ti + 2 * d * off[a]];
                             } else {
+                                int bx, by, bz;
+                                brick_at(g, b, bx, by, bz);
                                 const long long nb = brick_next(g, bx, by, bz, 2 * a + (d > 0 ? 1 : 0));
                                 if (nb >= 0) {
                                     const int step_c = a == 0 ? 1 : (a == 1 ? 8 : 64);
@@ -702,9 +734,8 @@ __global__ void __launch_bounds__(kStepWarps * 32)
                     if (blt(r, Tc))
                         next[base + c] = r;
                 }
-                __syncwarp();
+                __syncthreads();
             }
-            __syncthreads();
         }
         target += gridDim.x;
         run = grid_barrier(barrier, target, ctrl);
@@ -881,7 +912,7 @@ template <typename real, int kAcc>
 cudaError_t steps_t(const Geom &g, const DeviceState &s, const SolveParams &p, void *next, unsigned long long *mins,
                     long long step, int n, cudaStream_t st)
 {
-    const size_t sm = sizeof(StepTile<real>) * kStepWarps;
+    const size_t sm = sizeof(StepSmem<real>);
     int dev = 0, sms = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e == cudaSuccess)
@@ -891,8 +922,7 @@ cudaError_t steps_t(const Geom &g, const DeviceState &s, const SolveParams &p, v
     if (e != cudaSuccess)
         return e;
     // one CTA per SM (the barrier costs with every CTA), no more than there are bricks
-    const long long need = (g.nbricks + kStepWarps - 1) / kStepWarps;
-    const int nb = (int)(need < sms ? need : sms);
+    const int nb = (int)(g.nbricks < sms ? g.nbricks : sms);
     unsigned *barrier = (unsigned *)(mins + 4);
     e = cudaMemsetAsync(barrier, 0, sizeof(unsigned), st);
     if (e != cudaSuccess)
