@@ -244,6 +244,10 @@ fmm_status load_speed(fmm_handle *hd, const void *speed, double speed_const)
             hd->params.spd_term = (double)((hf * hf) / (F * F));
         }
     }
+    int dev = 0, sms = 0;
+    FMM_CUDA(hd, cudaGetDevice(&dev));
+    FMM_CUDA(hd, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
+    hd->params.raise_at = raise_threshold(s.march_ctas, s.spd && hd->params.aniso && hd->cfg.dtype == FMM_F64, sms);
     hd->tape_valid = false;
     hd->resumable = false;
     return FMM_OK;
@@ -735,7 +739,6 @@ fmm_status fmm_create(const fmm_config *cfg, const void *speed, double speed_con
         return bail(cuda_fail(hd, e, "cudaMallocHost"));
     const int per_sm = march_blocks_per_sm(cfg->dtype, cfg->record_tape != 0);
     s.march_ctas = cfg->ctas > 0 ? cfg->ctas : march_grid(sms * per_sm, g.nbricks);
-    hd->params.raise_at = raise_threshold(s.march_ctas);
     fmm_status rc = load_speed(hd, speed, speed_const);
     if (rc != FMM_OK)
         return bail(rc);

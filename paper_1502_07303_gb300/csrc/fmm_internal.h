@@ -153,7 +153,16 @@ constexpr int kMarchWarps = 4;   // bricks in flight per CTA of the march kernel
 // Continuous schedule: the bound rises once fewer bricks than this are queued
 // or marching: the warps of the march launch (half of them left 30% of the
 // 1024^3 march's warp time idle: 65 against 55 ms; twice as many: the same)
-inline int raise_threshold(int march_ctas) { return march_ctas * kMarchWarps; }
+// With a speed field and unequal cells in double the march runs on the FP64 pipe,
+// and bricks started ahead of the front, to be marched again, take it from those
+// at the front: there two bricks an SM (random speed, h = (1, 1.4, 0.7), one and 8
+// sources: 300^3 216 -> 59 and 130 -> 45 ms, 160^3 49 -> 27 and 31 -> 19, 64^3 and
+// below the same; one brick an SM 65, 49, 27.5, 18.7, four 61, 47, 34, 26)
+inline int raise_threshold(int march_ctas, bool fp64_pipe = false, int sms = 0)
+{
+    const int all = march_ctas * kMarchWarps;
+    return fp64_pipe && 2 * sms < all ? 2 * sms : all;
+}
 // CTAs of a march launch: as many as fit, but no more warps than bricks
 inline int march_grid(int full, long long nbricks)
 {

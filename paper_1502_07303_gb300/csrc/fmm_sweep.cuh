@@ -466,9 +466,9 @@ struct Notify {
 };
 
 // The cells to solve of a brick that marched before, to a lower bound: every cell
-// is the root of what was usable then, so they are the cells above a neighbour
-// that became usable (BAND, within the bound now) or above a halo value.  Marks
-// them.  (Not inlined: the march has no registers left for it.)
+// is the root of what was usable then (of the FIX cells before the first march),
+// so they are the cells above a neighbour that became usable (BAND, within the
+// bound now) or above a halo value.  Marks them.  (Not inlined: the march has no registers left for it.)
 template <typename real>
 __device__ __noinline__ void reopened_cells(const real *kv, const uint8_t *tg, unsigned *mark, int lane)
 {
@@ -608,7 +608,7 @@ __device__ __forceinline__ void sweep_brick(const Geom &g, const DeviceState &s,
         has_frozen = __any_sync(FULL, fr != 0u);
         was_known = __all_sync(FULL, (kn & 0x01010101u) == 0x01010101u);
         neg_side = __any_sync(FULL, ng != 0u);
-        if (kBounded && kHetero && sizeof(real) == 8)
+        if (kBounded && kHetero && !kAniso && sizeof(real) == 8)
             marched = __any_sync(FULL, mk != 0u);
     }
     __syncwarp();
@@ -720,8 +720,11 @@ __device__ __forceinline__ void sweep_brick(const Geom &g, const DeviceState &s,
     // restart per level (schedule 2), 160^3 with 8 sources 36.2 ms when such bricks
     // are swept, 27.6 so, 24^3 with one 3.95 and 3.0 (the bucketed march: 29.8 and
     // 3.45).  Without a speed field or in float a front runs straight through and
-    // sweeps win: 200^3 in double, phased, 18.2 ms swept, 20.0 so.
-    if (kBounded && kHetero && sizeof(real) == 8 && marched && !was_known) {
+    // sweeps win: 200^3 in double, phased, 18.2 ms swept, 20.0 so.  With unequal
+    // cells as well a solve itself runs on the FP64 pipe, and every march starts so
+    // (before the first one FIX cells have been used by Algorithm 9): 24^3, one
+    // source, 4.0 ms when a first march sweeps, 3.6 so.
+    if (kHetero && sizeof(real) == 8 && (kAniso || (kBounded && marched)) && !was_known) {
         reopened_cells<real>(W.kv, W.tg, W.mark, lane);
         __syncwarp();
         cells = W.mark[lane];
