@@ -505,6 +505,16 @@ fmm_status fmm_selftest_root(const double *m, const double *v1, const double *v2
                              const double *q, double *t_out, int32_t *k_out, int64_t n, void *stream);
 
 /*
+ * fmm_selftest_root_forward -- the same for the root as a march without a
+ * recorded tape computes it: the causal set is chosen in float, so within a
+ * few float ulp of a tie k_out may be the other set, whose root agrees to
+ * about 1e-13 of the shift.
+ */
+fmm_status fmm_selftest_root_forward(const double *m, const double *v1, const double *v2, const int32_t *nd,
+                                     const double *q, double *t_out, int32_t *k_out, int64_t n,
+                                     void *stream);
+
+/*
  * fmm_probe_fma_rate -- diagnostics: the device's fused multiply-add
  * throughput in float (dtype FMM_F32) or double (FMM_F64), the arithmetic
  * ceiling the march kernels are held to beside HBM bandwidth (on GB300 the

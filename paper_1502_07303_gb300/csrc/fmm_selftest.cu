@@ -42,10 +42,12 @@ extern "C" fmm_status fmm_selftest_fp64(const double *a, const double *b, double
 // ---------------------------------------------------------------------------
 // The double-grid root of Algorithm 11 (fmm_df.cuh's df_root) on
 // caller arrays: sorted upwind values m <= v1 <= v2 (nd of them used), speed
-// term q; returns the root and the size of the causal set it chose.
+// term q; returns the root and the size of the causal set it chose.  kStrict: as
+// the march computes it when it records the upwind sets, else as without.
 // ---------------------------------------------------------------------------
 namespace {
 
+template <bool kStrict>
 __global__ void k_selftest_root(const double *__restrict__ m, const double *__restrict__ v1,
                                 const double *__restrict__ v2, const int *__restrict__ nd,
                                 const double *__restrict__ q, double *__restrict__ t_out,
@@ -54,20 +56,17 @@ __global__ void k_selftest_root(const double *__restrict__ m, const double *__re
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n;
          i += (long long)gridDim.x * blockDim.x) {
         double t = 0.0;
-        // as the march computes it when it records the upwind sets
         const double inf = __longlong_as_double(0x7ff0000000000000ll);
-        const int k = fmmgb::df_root<true>(m[i], nd[i] >= 2 ? v1[i] : inf, nd[i] >= 3 ? v2[i] : inf,
-                                             fmmgb::df_speed(q[i]), q[i], t);
+        const int k = fmmgb::df_root<kStrict>(m[i], nd[i] >= 2 ? v1[i] : inf, nd[i] >= 3 ? v2[i] : inf,
+                                              fmmgb::df_speed(q[i]), q[i], t);
         t_out[i] = k ? t : __longlong_as_double(0x7ff0000000000000ll);
         k_out[i] = k;
     }
 }
 
-}  // namespace
-
-extern "C" fmm_status fmm_selftest_root(const double *m, const double *v1, const double *v2,
-                                        const int32_t *nd, const double *q, double *t_out,
-                                        int32_t *k_out, int64_t n, void *stream)
+template <bool kStrict>
+fmm_status selftest_root(const double *m, const double *v1, const double *v2, const int32_t *nd, const double *q,
+                         double *t_out, int32_t *k_out, int64_t n, void *stream)
 {
     if (n < 0 || (n > 0 && (!m || !v1 || !v2 || !nd || !q || !t_out || !k_out)))
         return FMM_ERR_INVALID;
@@ -76,9 +75,25 @@ extern "C" fmm_status fmm_selftest_root(const double *m, const double *v1, const
     long long blocks = (n + 255) / 256;
     if (blocks > 152 * 16)
         blocks = 152 * 16;
-    k_selftest_root<<<(int)blocks, 256, 0, (cudaStream_t)stream>>>(m, v1, v2, (const int *)nd, q, t_out,
-                                                                 (int *)k_out, n);
+    k_selftest_root<kStrict><<<(int)blocks, 256, 0, (cudaStream_t)stream>>>(m, v1, v2, (const int *)nd, q, t_out,
+                                                                          (int *)k_out, n);
     return cudaGetLastError() == cudaSuccess ? FMM_OK : FMM_ERR_CUDA;
+}
+
+}  // namespace
+
+extern "C" fmm_status fmm_selftest_root(const double *m, const double *v1, const double *v2,
+                                        const int32_t *nd, const double *q, double *t_out,
+                                        int32_t *k_out, int64_t n, void *stream)
+{
+    return selftest_root<true>(m, v1, v2, nd, q, t_out, k_out, n, stream);
+}
+
+extern "C" fmm_status fmm_selftest_root_forward(const double *m, const double *v1, const double *v2,
+                                                const int32_t *nd, const double *q, double *t_out,
+                                                int32_t *k_out, int64_t n, void *stream)
+{
+    return selftest_root<false>(m, v1, v2, nd, q, t_out, k_out, n, stream);
 }
 
 // ---------------------------------------------------------------------------
