@@ -1,22 +1,24 @@
-// fmm_df.cuh -- the root of Algorithm 11 for double-precision grids, computed
-// in double-float arithmetic (a value is an unevaluated sum hi + lo of two
-// floats, about 46 significant bits) so that the FP64 pipe, which on GB300
-// runs at 1/64 of the float rate, only does the four additions whose
-// operands are of order psi: the two shifts delta_i = psi_i - m, the
-// recombination of the root u, and t = m + u.  Everything of order h (the
-// shifted values, the speed term, the discriminant, its square root and u)
-// lives in the float pipe.
+// fmm_df.cuh -- the root of Algorithm 11 for double-precision grids with as
+// little as possible on the FP64 pipe, which on GB300 runs at 1/64 of the float
+// rate.
+//
+// df_root takes three FP64 additions, the ones whose operands are of order psi:
+// the two shifts delta_i = psi_i - m and t = m + u.  The upwind set and a first
+// root come from float arithmetic, then the exact residual of the quadratic about
+// that root, in double-float (a value is an unevaluated sum hi + lo of two floats,
+// about 46 significant bits), gives the correction.  Where the upwind set is
+// recorded and a test is too close for float, df_shifted_root carries the whole
+// root in double-float instead (four FP64 additions) and decides on the doubles.
 //
 // Error-free transformations (Knuth's two-sum, Dekker's fast two-sum, the
 // exact product a*b - fl(a*b) from one fused multiply-add) build the
-// double-float sums and products; the square root takes a float estimate
-// x * rsqrt(x) and one Newton step carried in double-float.
+// double-float sums and products.
 //
 // Accuracy: for a causal root the discriminant is at least q/2 (q the speed
-// term (h/F)^2), so no step cancels catastrophically and u carries a
-// relative error of a few 1e-14, i.e. ~1e-16 absolute on a grid with
-// h = 1/1024: far below the fp64 parity tolerance of 1e-12 max|psi| even
-// summed along a path of a thousand cells.
+// term (h/F)^2), so no step cancels catastrophically and u carries a relative
+// error of at most 3e-14 (against exact arithmetic, ties included), i.e. ~3e-17
+// absolute on a grid with h = 1/1024: far below the fp64 parity tolerance of
+// 1e-12 max|psi| even summed along a path of a thousand cells.
 #pragma once
 
 #include "fmm_fp64.cuh"
@@ -82,21 +84,12 @@ __device__ __forceinline__ dfl df_sqrt(dfl x)
     return df_fast_two_sum(s, res * (0.5f * r));
 }
 
-// x < y for normalized pairs (|l| at most half an ulp of h, as the
-// operations above return them): then the high parts decide unless they are
-// equal
-__device__ __forceinline__ bool df_lt(dfl x, dfl y)
-{
-    return x.h < y.h || (x.h == y.h && x.l < y.l);
-}
-
 // A non-negative double of magnitude below 1e30 as a double-float: the value
 // truncated to 24 significant bits (fmm_fp64.cuh's f32_of) plus the remaining
 // fraction bits as a float (the low 29 bits of the double's fraction, of which
 // the top 23 are kept), both built with integer operations.  The pair is not
-// normalized (lo may reach a whole ulp of hi), so df_lt against it can order
-// two values wrongly when they lie within a float ulp of each other.  Values below 2^-100 become 0 (an absolute error no Algorithm
-// 11 operand of order h notices).
+// normalized (lo may reach a whole ulp of hi).  Values below 2^-100 become 0 (an
+// absolute error no Algorithm 11 operand of order h notices).
 __device__ __forceinline__ dfl df_of(double v)
 {
     const unsigned long long b = (unsigned long long)__double_as_longlong(v);
@@ -126,12 +119,10 @@ __device__ __forceinline__ double df_to_double(dfl x)
 // With delta_i = v_i - m the root is t = m + u, u the larger root of
 // sum_i (u - delta_i)^2 = q over the set: u = (S + sqrt(k q - P)) / k with
 // S = sum delta_i and P = sum_{i<j} (delta_i - delta_j)^2 (Lagrange's form of
-// S^2 - k (Q - q), a sum of squares, so nothing cancels), causal when the
-// largest delta is below u (kStrict: when the double root t = m + u exceeds
-// the largest value); the largest value is dropped while the set is not
-// causal.  Returns the number of values in the causal set (0: none, root
-// +inf) and the root in t.
-template <bool kStrict>
+// S^2 - k (Q - q), a sum of squares, so nothing cancels), causal when the double
+// root t = m + u exceeds the largest value; the largest value is dropped while
+// the set is not causal.  Returns the number of values in the causal set (0:
+// none, root +inf) and the root in t.
 __device__ __forceinline__ int df_shifted_root(double m, double v1, double v2, int nd, double q,
                                                double &t)
 {
@@ -156,29 +147,15 @@ __device__ __forceinline__ int df_shifted_root(double m, double v1, double v2, i
         if (disc.h > 0.0f) {
             const dfl r = df_add(S, df_sqrt(disc));
             const dfl u = nd == 3 ? df_mul(r, third) : (nd == 2 ? dfl{0.5f * r.h, 0.5f * r.l} : r);
-            if constexpr (kStrict) {
-                // causal when the root exceeds the largest value of the set,
-                // tested on the doubles the cell and its neighbours will hold
-                // (the test on the shifted double-floats can pass by a
-                // rounding step while t rounds to that value or below it; an
-                // upwind set recorded for the adjoint must point strictly
-                // downhill)
-                const double tt = m + df_to_double(u);
-                const double vmax = nd == 3 ? v2 : v1;
-                if (nd == 1 || __double_as_longlong(vmax) < __double_as_longlong(tt)) {
-                    t = tt;
-                    return nd;
-                }
-            } else {
-                // without a recorded set, the shifted test suffices: it can
-                // err only where u and the largest delta lie within a float
-                // ulp of each other, and there the two sets' roots agree to
-                // about 1e-14 u
-                const dfl dmax = nd == 3 ? D2 : D1;   // 0 when nd == 1
-                if (df_lt(dmax, u)) {
-                    t = m + df_to_double(u);
-                    return nd;
-                }
+            // (tested on the doubles the cell and its neighbours will hold: the
+            // test on the shifted double-floats can pass by a rounding step while
+            // t rounds to that value or below it, and an upwind set recorded for
+            // the adjoint must point strictly downhill)
+            const double tt = m + df_to_double(u);
+            const double vmax = nd == 3 ? v2 : v1;
+            if (nd == 1 || __double_as_longlong(vmax) < __double_as_longlong(tt)) {
+                t = tt;
+                return nd;
             }
         }
         if (nd == 3)
@@ -260,7 +237,7 @@ __device__ __forceinline__ DfSpeed df_speed(double q)
 //
 // With r = q - sum (u0 - delta_i)^2 in double-float and g = sum (u0 -
 // delta_i), u - u0 = c - k c^2 / (2 g) + O(c^3), c = r / (2 g); c is about 1e-7
-// u0, so its float rounding is below 1e-14 u0.  Three FP64 additions in all
+// u0, so its float rounding is about 1e-14 u0 (all in all at most 3e-14).  Three FP64 additions in all
 // (two shifts and m + u) on a pipe that takes one warp instruction in 16
 // cycles, against four, and about half the float operations, when the root is
 // carried in double-float throughout (df_shifted_root).
@@ -274,7 +251,7 @@ __device__ __forceinline__ int df_root(double m, double v1, double v2, const DfS
     const bool c2 = a2 < u2;
     if constexpr (kStrict) {
         if (fabsf(a1 - Q.s) < 1e-5f * Q.s || (c1 && fabsf(a2 - u2) < 1e-5f * u2))
-            return df_shifted_root<true>(m, v1, v2, v1 < 1e300 ? (v2 < 1e300 ? 3 : 2) : 1, q, t);
+            return df_shifted_root(m, v1, v2, v1 < 1e300 ? (v2 < 1e300 ? 3 : 2) : 1, q, t);
     }
     // (products that feed an error-free sum are rounded on their own: a fused
     // multiply-add there would not be the sum whose error is taken)
@@ -308,7 +285,7 @@ __device__ __forceinline__ int df_root(double m, double v1, double v2, const DfS
     if constexpr (kStrict) {
         // m so large that t rounds to a value of the set
         if (c1 && __double_as_longlong(t) <= __double_as_longlong(c2 ? v2 : v1))
-            return df_shifted_root<true>(m, v1, v2, v1 < 1e300 ? (v2 < 1e300 ? 3 : 2) : 1, q, t);
+            return df_shifted_root(m, v1, v2, v1 < 1e300 ? (v2 < 1e300 ? 3 : 2) : 1, q, t);
     }
     return c2 ? 3 : (c1 ? 2 : 1);
 }
