@@ -4,9 +4,8 @@ The paper's only free parameter is the restart stride (Sec. 4.4, Sec. 5.1):
 it studies 0.5-3.5 h and infinity, suggests 2 h for its CPU cluster and
 advises experimenting on new platforms (Sec. 5.5).  On the GPU the stride,
 the restart schedule (continuous, persistent queue or phased passes), the
-look-ahead of a brick march beyond the bound, the bucket width of the local
-march, the number of exchange passes per restart (phased schedule) and the
-number of CTAs of the march kernel all trade restarts against
+look-ahead of a brick march beyond the bound, the number of exchange passes per
+restart (phased schedule) and the number of CTAs of the march kernel all trade restarts against
 re-acceptance, so they are tuned together.  The brick is 8x8x8 (one warp per
 brick, a 16-bit cell mask per lane); the CTA count sets how many bricks march
 at once.
@@ -34,7 +33,7 @@ PARAMS = ("schedule", "stride", "bucket", "exchange_passes", "ctas", "max_lead",
 SEARCH = {
     "schedule": [1, 2, 3],
     "stride": [0.5, 1.0, 2.0, 4.0, 8.0, math.inf],
-    "bucket": [2.0, 3.0, 4.0, 6.0],
+    "bucket": [0.0],   # the brick schedules take no bucket
     "exchange_passes": [1, 2],
     "ctas": [0, 152 * 2, 152 * 4],
     "max_lead": [0],
@@ -42,15 +41,12 @@ SEARCH = {
 }
 
 # A short list for a quick tune: the continuous schedule with a whole-brick
-# look-ahead over strides and bucket widths (around the fp64 optimum of 1 h
-# and the fp32 one of 2 h), at the full and at a reduced CTA count, and the
-# persistent schedule without restarts.
-QUICK = ([{"schedule": 3, "stride": s, "bucket": 4.0, "ahead": math.inf}
-          for s in (0.5, 1.0, 1.5, 2.0, 3.0, 4.0)]
-         + [{"schedule": 3, "stride": 1.0, "bucket": b, "ahead": math.inf} for b in (5.0, 6.0)]
-         + [{"schedule": 3, "stride": 2.0, "bucket": b, "ahead": math.inf} for b in (3.0, 6.0)]
-         + [{"schedule": 3, "stride": 1.0, "bucket": 4.0, "ahead": math.inf, "ctas": 152 * 4}]
-         + [{"schedule": 2, "stride": math.inf, "bucket": 4.0}])
+# look-ahead over strides (around the fp64 optimum of 1 h and the fp32 one of
+# 2 h), at the full and at a reduced CTA count, and the persistent schedule without
+# restarts.
+QUICK = ([{"schedule": 3, "stride": s, "ahead": math.inf} for s in (0.5, 1.0, 1.5, 2.0, 3.0, 4.0)]
+         + [{"schedule": 3, "stride": 1.0, "ahead": math.inf, "ctas": 152 * 4}]
+         + [{"schedule": 2, "stride": math.inf}])
 
 
 def cache_path(path=None):
