@@ -58,14 +58,29 @@ def peaks():
         return 6800.0, "fallback"
 
 
+# the source of the march kernels: scheduler, sweep, root and its arithmetic
+MARCH_SOURCES = ("fmm_march.cu", "fmm_sweep.cuh", "fmm_df.cuh", "fmm_fp64.cuh", "fmm_queue.cuh", "fmm_ring.h")
+
+
+def march_source_sha():
+    """First 16 hex digits of the sha256 over those of MARCH_SOURCES that the
+    tree has, one after another."""
+    h = hashlib.sha256()
+    for name in MARCH_SOURCES:
+        path = os.path.join(ROOT, "paper_1502_07303_gb300", "csrc", name)
+        if os.path.exists(path):
+            with open(path, "rb") as f:
+                h.update(f.read())
+    return h.hexdigest()[:16]
+
+
 def _profile_record(fname, kernel, dtype, workload):
     """A per-point figure of a march kernel from a committed ncu summary
-    (lines "kernel dtype workload source_sha256_16 value"), valid only while
-    the kernel source is unchanged."""
+    (lines "march dtype workload source_sha256_16 value"), valid only while
+    the march's sources are unchanged."""
     path = os.path.join(ROOT, "profiles", fname)
-    src = os.path.join(ROOT, "paper_1502_07303_gb300", "csrc", "fmm_march.cu")
     try:
-        sha = hashlib.sha256(open(src, "rb").read()).hexdigest()[:16]
+        sha = march_source_sha()
         for line in open(path):
             f = line.split()
             if len(f) == 5 and not line.startswith("#") and f[0] == kernel and f[1] == dtype \
@@ -533,6 +548,10 @@ def tune_params(autotune, torch, p, dt, stream, kind, search=None):
     return best or {}, [[c, None if ms is None else round(ms, 3)] for c, ms in table]
 
 
+# the kernel that runs a march the profile records name
+KERNELS = {"k_march_continuous": "k_march_queue", "k_march_persistent": "k_march_queue"}
+
+
 def roofline_hbm(r, pts, alg, kernel, dt, workload, peak, peak_kind):
     """HBM roofline of the dominant kernel: algorithmic bytes of one launch
     over its average CUDA-event duration, against the measured copy peak."""
@@ -542,7 +561,7 @@ def roofline_hbm(r, pts, alg, kernel, dt, workload, peak, peak_kind):
     bpp = traffic_record(kernel, dt, workload)
     return {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak, "traffic": (bpp * pts / launches) if bpp else None,
-            "kernel": kernel, "peak_kind": peak_kind, "alg_bytes_per_point": alg,
+            "kernel": KERNELS.get(kernel, kernel), "peak_kind": peak_kind, "alg_bytes_per_point": alg,
             "avg_launch_us": 1e3 * r["march_ms"] / launches,
             "launches_per_step": r["march_launches"], "share_of_step": r["march_ms"] / r["ms"]}
 
@@ -561,7 +580,7 @@ def roofline_alu(r, pts, kernel, dt, workload, fp64_peak, sms, sm_mhz):
     peak = 4 * sms * sm_mhz * 1e6 / 1e12
     ach = per_pt * pts / launches / avg_s / 1e12 if (per_pt and avg_s > 0) else None
     out = {"bound": "alu", "pipe": "issue", "achieved": ach, "peak": peak, "unit": "Tinst/s",
-           "frac": (ach / peak) if ach else None, "kernel": kernel,
+           "frac": (ach / peak) if ach else None, "kernel": KERNELS.get(kernel, kernel),
            "peak_kind": f"derived: 4 warp instructions per clock per SM x {sms} SMs x {sm_mhz:.0f} MHz",
            "ops_per_point": per_pt}
     if dt == "f64":
@@ -576,8 +595,7 @@ def roofline_alu(r, pts, kernel, dt, workload, fp64_peak, sms, sm_mhz):
 
 
 def kernel_name(params):
-    """The march of a schedule as the profile records name it (the continuous
-    and the persistent one are k_march_queue)."""
+    """The march of a schedule as the profile records name it."""
     return {1: "k_march", 2: "k_march_persistent"}.get(params.get("schedule", 0), "k_march_continuous")
 
 

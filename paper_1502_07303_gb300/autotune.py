@@ -5,8 +5,8 @@ it studies 0.5-3.5 h and infinity, suggests 2 h for its CPU cluster and
 advises experimenting on new platforms (Sec. 5.5).  On the GPU the stride,
 the restart schedule (continuous, persistent queue or phased passes), the
 look-ahead of a brick march beyond the bound, the number of exchange passes per
-restart (phased schedule) and the number of CTAs of the march kernel all trade restarts against
-re-acceptance, so they are tuned together.  The brick is 8x8x8 (one warp per
+restart (phased schedule) and the number of CTAs of the march kernel all trade
+restarts against re-acceptance, so they are tuned together.  The brick is 8x8x8 (one warp per
 brick, a 16-bit cell mask per lane); the CTA count sets how many bricks march
 at once.
 

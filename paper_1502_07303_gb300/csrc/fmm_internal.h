@@ -220,7 +220,7 @@ struct DeviceState {
     int *list[2];       // work lists
     const int *nbr;     // 6 per brick: neighbour brick or -1 (batches only)
     unsigned long long *queue;   // persistent march: ring of (seq << 32 | brick + 1)
-    unsigned *queued;            // per brick: in the queue or being marched
+    unsigned *queued;            // per brick: in the queue (the adjoint; null without a handle)
     Control *ctrl;
     int march_ctas;
 };

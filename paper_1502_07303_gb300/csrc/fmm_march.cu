@@ -462,9 +462,9 @@ __global__ void __launch_bounds__(kThreads) k_load_speed(Geom g, double h, doubl
 // The brick march (fmm_sweep.cuh): one warp per brick, four bricks per CTA.  It
 // is bound by the length of a brick's chain of steps where a grid has few
 // bricks per warp, and by the ALU (float) and FP64 (double) pipes where it has
-// many.  256^3 level set of 32 spheres, whole call: 1.8 ms in float, 4.9 ms in
+// many.  256^3 level set of 32 spheres, whole call: 2.1 ms in float, 5.0 ms in
 // double (5.7 and 12.0 ms with the bucketed march this replaced); 1024^3 sphere
-// in double 59 ms (236 ms).
+// in double 55 ms (236 ms).
 // ---------------------------------------------------------------------------
 
 #ifndef FMM_MARCH_BLOCKS_F32
@@ -476,10 +476,10 @@ __global__ void __launch_bounds__(kThreads) k_load_speed(Geom g, double h, doubl
 #ifndef FMM_MARCH_BLOCKS_F64_TAPE
 #define FMM_MARCH_BLOCKS_F64_TAPE 5
 #endif
-// Resident CTAs per SM the march kernels are compiled for (registers); the
-// warp tiles (5.7 / 6.2 KB in float, 9.7 / 10.2 KB in double, without / with
-// the tape) allow these as well.  Six fp64 CTAs would leave 80 registers and
-// spill.
+// Resident CTAs per SM the march kernels are compiled for (registers).  The warp
+// tiles (5.7 / 6.2 KB in float, 9.7 / 10.2 KB in double, without / with the tape)
+// and the sweep order (4 KB a CTA) allow these as well; six fp64 CTAs of 43 KB
+// would not fit the 227 KB of an SM.
 template <typename real, bool kTape>
 constexpr int march_min_blocks()
 {
@@ -681,7 +681,7 @@ __device__ __forceinline__ void finish_brick(const DeviceState &s, unsigned long
 // Phased march: kMode 0 runs Algorithm 9 over all bricks; kMode 1 runs
 // Algorithm 12 up to the restart bound over the bricks of work list `which`
 // (taken one at a time from a shared counter); changes are flagged in the
-// neighbours' live masks and dirty flags.
+// neighbours' dirty flags.
 template <typename real, bool kHetero, int kMode, bool kTape, bool kAniso>
 __global__ void __launch_bounds__(kMarchWarps * 32, march_min_blocks<real, kTape>())
     k_march(Geom g, DeviceState s, SolveParams p, double spd_const_term, int which)
@@ -1575,7 +1575,7 @@ size_t march_smem() { return sizeof(MarchSmem<real, kTape>); }
 
 // Deterministic mode: face f of brick b is its boundary layer on side f
 // (0..5 = -x, +x, -y, +y, -z, +z), cell q = u + 8 v in the in-face
-// coordinates of the halo loader of march_brick, holding the known value or
+// coordinates of the halo loader of sweep_brick, holding the known value or
 // +inf.  A march pass reads its neighbours' faces and the faces of the bricks
 // it marched are rebuilt after the pass (which >= 0: work list `which`), so
 // a pass sees the state of the previous one whatever the order of its

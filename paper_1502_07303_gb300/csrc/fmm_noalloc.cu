@@ -55,8 +55,7 @@ constexpr size_t kOffDirty = align256(kOffWaiting + waiting_slots(kNoAllocMaxBri
 constexpr size_t kOffList0 = align256(kOffDirty + kNoAllocMaxBricks * sizeof(unsigned));
 constexpr size_t kOffList1 = align256(kOffList0 + kNoAllocMaxBricks * sizeof(int));
 constexpr size_t kOffQueue = align256(kOffList1 + kNoAllocMaxBricks * sizeof(int));
-constexpr size_t kOffQueued = align256(kOffQueue + kNoAllocMaxBricks * sizeof(unsigned long long));
-constexpr size_t kOffCtrl = align256(kOffQueued + kNoAllocMaxBricks * sizeof(unsigned));
+constexpr size_t kOffCtrl = align256(kOffQueue + kNoAllocMaxBricks * sizeof(unsigned long long));
 constexpr size_t kScratchBytes = align256(kOffCtrl + sizeof(Control));   // about 2.4 MiB
 
 __device__ __align__(256) unsigned char g_noalloc_scratch[kScratchBytes];
@@ -173,7 +172,6 @@ extern "C" fmm_status fmm_reinit_signed_distance_noalloc(const fmm_config *cfg, 
     s.list[0] = (int *)(base + kOffList0);
     s.list[1] = (int *)(base + kOffList1);
     s.queue = (unsigned long long *)(base + kOffQueue);
-    s.queued = (unsigned *)(base + kOffQueued);
     s.ctrl = (Control *)(base + kOffCtrl);
     s.spd = nullptr;
     s.tape = nullptr;
@@ -219,7 +217,6 @@ extern "C" fmm_status fmm_reinit_signed_distance_noalloc(const fmm_config *cfg, 
     NA_CUDA(cudaMemsetAsync(s.waiting, 0, waiting_bytes(g.nbricks), st));
     NA_CUDA(cudaMemsetAsync(s.dirty, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     NA_CUDA(cudaMemsetAsync(s.queue, 0, (size_t)g.nbricks * sizeof(unsigned long long), st));
-    NA_CUDA(cudaMemsetAsync(s.queued, 0, (size_t)g.nbricks * sizeof(unsigned), st));
     NA_CUDA(launch_load_speed(dt, g, s, p.h, min_spacing(p), nullptr, 1.0, st));
     NA_CUDA(launch_init_reinit(dt, g, s, p, phi0, st));
     NA_CUDA(launch_front_init(dt, g, s, p, st));
