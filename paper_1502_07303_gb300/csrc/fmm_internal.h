@@ -178,8 +178,9 @@ inline bool one_launch_schedule(int schedule)
 // measured on GB300 for 8^3 bricks.
 inline double default_stride(int dtype) { return dtype == 1 ? 1.0 : 2.0; }
 // deterministic mode (phased schedule, pass-synchronous halos): information
-// crosses one brick per pass, so wider strides pay (1024^3 sphere: fp64
-// 722 / 493 / 529 ms at 1 / 4 / 8 h, fp32 374 / 278 / 238 ms at 2 / 4 / 8 h)
+// crosses one brick per pass, so wider strides pay (1024^3 sphere, with the
+// bucketed brick march: fp64 722 / 493 / 529 ms at 1 / 4 / 8 h, fp32 374 / 278 /
+// 238 ms at 2 / 4 / 8 h)
 inline double default_stride_deterministic(int dtype) { return dtype == 1 ? 4.0 : 8.0; }
 inline int default_passes(int dtype) { return dtype == 1 ? 1 : 2; }
 // continuous schedule: look-ahead of a brick march beyond the bound (units of
