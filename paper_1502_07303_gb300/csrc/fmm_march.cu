@@ -1737,9 +1737,9 @@ cudaError_t front_init_impl(const Geom &g, const DeviceState &s, const SolvePara
     return cudaGetLastError();
 }
 
-// Shared-memory attributes of every march kernel; returns the resident CTAs
-// per SM of the march kernels with or without the tape (the smallest over
-// the kernels a solve may launch).
+// Shared-memory attributes of the march kernels with or without the tape;
+// returns their resident CTAs per SM (the smallest over the kernels a solve may
+// launch).
 template <typename real>
 int configure_march(bool tape)
 {
@@ -1748,14 +1748,14 @@ int configure_march(bool tape)
     for (int f = 0; f < 8; ++f)
         with_flags((f & 1) != 0, (f & 2) != 0, (f & 4) != 0, [&](auto H, auto P, auto A) {
             constexpr bool hh = decltype(H)::value, tt = decltype(P)::value, an = decltype(A)::value;
+            if (tt != tape)   // (a handle launches the kernels with or without the tape, never both)
+                return;
             const int sm = (int)march_smem<real, tt>();
             cudaFuncSetAttribute(k_march<real, hh, 1, tt, an>, attr, sm);
             cudaFuncSetAttribute(k_march<real, hh, 0, tt, an>, attr, sm);
             cudaFuncSetAttribute(k_march_queue<real, hh, tt, an, true, true>, attr, sm);
             cudaFuncSetAttribute(k_march_queue<real, hh, tt, an, true, false>, attr, sm);
             cudaFuncSetAttribute(k_march_queue<real, hh, tt, an, false, false>, attr, sm);
-            if (tt != tape)
-                return;
             int k = 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&k, k_march_queue<real, hh, tt, an, false, false>,
                                                           kMarchWarps * 32, sm);
